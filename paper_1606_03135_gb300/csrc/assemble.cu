@@ -1801,20 +1801,37 @@ __global__ void __launch_bounds__(256) k_finalize(SolveArgs a, long long* __rest
     }
 }
 
-// y = L u, one warp per row
+// y = L u, kSpmvLanes lanes per row.  An FP64 warp instruction takes 16 cycles of the SM's FP64
+// units however many lanes it uses, so a whole warp per row was bound by its reduction: two FMAs
+// and five shuffle-adds per row of 45 entries, 36 us of FP64 issue for N = 100,000 (53 us in all,
+// against 8 us for the matrix's bytes).  Four lanes per row take 12 FMAs and two adds for eight
+// rows, 9 us.  Each lane keeps four entries in flight (values, columns, then the gathers of u):
+// 20.6 us, the latency of the gathers and the loads of the matrix.
+constexpr int kSpmvLanes = 4;
 __global__ void __launch_bounds__(256) k_spmv(int N, const long long* __restrict__ row_ptr,
                                               const int* __restrict__ col,
                                               const double* __restrict__ val,
                                               const double* __restrict__ u, double* __restrict__ y) {
-    const int lane = threadIdx.x & 31;
-    const int wpb = blockDim.x >> 5;
-    for (int i = blockIdx.x * wpb + (threadIdx.x >> 5); i < N; i += gridDim.x * wpb) {
-        const long long b = row_ptr[i], e = row_ptr[i + 1];
-        double s = 0.0;
-        for (long long k = b + lane; k < e; k += 32) s = fma(val[k], __ldg(&u[col[k]]), s);
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (lane == 0) y[i] = s;
+    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const int l = (int)(t & (kSpmvLanes - 1));
+    const int i = (int)min(t / kSpmvLanes, (long long)N - 1);  // (whole warps reach the shuffles)
+    const long long b = row_ptr[i], e = row_ptr[i + 1];
+    double s = 0.0;
+    for (long long k = b + l; k < e; k += 4 * kSpmvLanes) {
+        double v[4], x[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const long long kk = k + j * kSpmvLanes;
+            const bool in = kk < e;
+            v[j] = in ? __ldg(&val[kk]) : 0.0;
+            x[j] = in ? __ldg(&u[__ldg(&col[kk])]) : 0.0;
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (k + j * kSpmvLanes < e) s = fma(v[j], x[j], s);
     }
+    for (int o = kSpmvLanes / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (l == 0 && t / kSpmvLanes < N) y[i] = s;
 }
 
 // Values of the time-stepping matrix of §5 on L's pattern, one warp per row: interior rows
@@ -2140,9 +2157,9 @@ int launch_timestep(int N, const long long* row_ptr, const int* col, const doubl
 int launch_spmv(int N, int n, const long long* row_ptr, const int* col, const double* val,
                 const double* u, double* y, cudaStream_t s, int* launches) {
     (void)n;
-    const int wpb = 8;
-    const int blocks = (N + wpb - 1) / wpb;
-    k_spmv<<<blocks, wpb * 32, 0, s>>>(N, row_ptr, col, val, u, y);
+    const int tb = 256;
+    const unsigned blocks = (unsigned)(((long long)N * kSpmvLanes + tb - 1) / tb);
+    k_spmv<<<blocks, tb, 0, s>>>(N, row_ptr, col, val, u, y);
     ++*launches;
     return RB_LAUNCHED(__func__);
 }

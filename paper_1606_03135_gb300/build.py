@@ -17,7 +17,7 @@ CSRC = os.path.join(HERE, "csrc")
 OUT_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT_DIR, "librbffd.so")
 PROBE_LIB = os.path.join(OUT_DIR, "libfp64probe.so")  # FP64 pipe probe (include/fp64_probe.h)
-SOURCES = ["knn.cu", "assemble.cu", "api.cu", "noalloc.cu"]
+SOURCES = ["assemble.cu", "nullspace.cu", "knn.cu", "api.cu", "noalloc.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",
          "--fmad=true", "-I", os.path.join(ROOT, "include")]

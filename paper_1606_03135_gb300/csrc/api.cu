@@ -55,6 +55,7 @@ struct rbffd_plan_s {
     long long total_slots = 0;
     int qcap = 0, stride = 0;
     LaunchPlan lp;
+    int lay = kLayPacked;           // layout of the local systems
     int refine_min_K = 0x7fffffff;  // systems with K >= this are refined
     long long rs_doubles = 0, rs_stride = 0;  // refinement scratch: size, per traversal CTA
     int rs_x0 = 0;                  // offset of the first solution within a slot
@@ -342,6 +343,7 @@ int plan_impl(const double* nodes, int64_t N, int d, int n, int ell, int m,
         !(delta <= 1.0))
         return RBFFD_EINVAL;
     const bool mixed = n_node != nullptr;
+    bool one_shape = true;  // every node has the same n, ell and m
     int ell_lo = ell, ell_hi = ell, K_max = n + (int)binom(ell + d, d);
     if ((int)binom(ell + d, d) > n) return RBFFD_EINVAL;
     if (mixed) {
@@ -354,9 +356,14 @@ int plan_impl(const double* nodes, int64_t N, int d, int n, int ell, int m,
                 return RBFFD_EINVAL;
             const int Mk = (int)binom(lk + d, d);
             if (Mk > nk) return RBFFD_EINVAL;
+            one_shape = one_shape && nk == n_node[0] && lk == ell_node[0] && mk == m_node[0];
             ell_lo = lk < ell_lo ? lk : ell_lo;
             ell_hi = lk > ell_hi ? lk : ell_hi;
             K_max = nk + Mk > K_max ? nk + Mk : K_max;
+        }
+        if (one_shape) {
+            ell = ell_node[0];
+            m = m_node[0];
         }
     }
     rbffd_opts o{RBFFD_STAB_SEQ, 0, 5000, 1, 0, RBFFD_FACTOR_LDLT, 0, 0, 0, RBFFD_LREF_CENTER,
@@ -506,11 +513,30 @@ int plan_impl(const double* nodes, int64_t N, int d, int n, int ell, int m,
         const size_t avail = (size_t)max_optin_smem() - 64;
         int stride = 0;
         size_t per_cta = 0;
-        for (;;) {
-            per_cta = solve_smem_per_cta(n, p->K, p->qcap, qmax, d, ldlt, &stride) +
-                      basis_smem_bytes((int)basis_count);
-            if (per_cta <= avail || !ldlt || p->qcap == 1) break;
-            --p->qcap;
+        p->refine_min_K = (!ldlt || o.refine == RBFFD_REFINE_NONE) ? 0x7fffffff
+                          : o.refine == RBFFD_REFINE_ALL           ? 0
+                                                                   : RBFFD_REFINE_MIN_K;
+        // Layouts to try.  LDL^T solves systems of one shape in the null space of the constraints
+        // when r^m is conditionally definite there (ell >= (m - 1) / 2) and the fixed-point forms
+        // are as accurate as the saddle-point factorization against a double-double solve: up to
+        // r^7 and degree 4 the norms of their errors are 0.3 to 1.0 times its over a set's rows.
+        // At degree 5 one-sided stencils are several times further off unless refined, as systems
+        // of K >= 100 are (2.6e-11 against the refined saddle-point solve's 2.6e-11); at degree 6
+        // and above (the constraints' pivots get small) and at r^9 and above (r^m spans more of the
+        // 58 bits) all are.  Refined systems with n > 3 M are left out as well: S is nearly the
+        // whole matrix there (n = 128, M = 21: 5.0 ms against 5.35).  Those, plans of several shapes
+        // and systems too large for this layout factor the saddle-point matrix.
+        const bool large = p->K >= RBFFD_REFINE_MIN_K;
+        const bool null_space = ldlt && one_shape && 2 * ell + 1 >= m && m <= 7 &&
+                                (large ? ell <= 5 && n <= 3 * (p->K - n) : ell <= 4);
+        const int qcap0 = p->qcap;
+        for (p->lay = null_space ? kLayNull : (ldlt ? kLayPacked : kLayFull);; p->lay = kLayPacked) {
+            for (p->qcap = qcap0;; --p->qcap) {
+                per_cta = solve_smem_per_cta(n, p->K, p->qcap, qmax, d, p->lay, &stride) +
+                          basis_smem_bytes((int)basis_count);
+                if (per_cta <= avail || !ldlt || p->qcap == 1) break;
+            }
+            if (per_cta <= avail || p->lay != kLayNull) break;
         }
         p->stride = stride;
         if (per_cta > avail) { rc = RBFFD_EINVAL; goto fail; }
@@ -533,11 +559,8 @@ int plan_impl(const double* nodes, int64_t N, int d, int n, int ell, int m,
                 }
         }
         p->lp.force_nt = o.team;
-        p->refine_min_K = (!ldlt || o.refine == RBFFD_REFINE_NONE) ? 0x7fffffff
-                          : o.refine == RBFFD_REFINE_ALL           ? 0
-                                                                   : RBFFD_REFINE_MIN_K;
         p->lp.refine_min_K = p->refine_min_K;
-        rc = prepare_solve_kernels(d, o.factor == RBFFD_FACTOR_LDLT, n, p->K, p->qcap, qmax,
+        rc = prepare_solve_kernels(d, p->lay, n, p->K, p->qcap, qmax,
                                    (int)basis_count, &p->lp);
         if (rc) goto fail;
         // refinement scratch: one slot per CTA of every launch that refines (the traversal when
@@ -547,14 +570,16 @@ int plan_impl(const double* nodes, int64_t N, int d, int n, int ell, int m,
             // per CTA: the full K x K matrix, then x0 and 4 partial sums per (unknown, column)
             auto sq32 = [](long long K) { return (K * K + 31) / 32 * 32; };
             const long long K = p->K;
+            const bool ns = p->lay == kLayNull;  // (its step: ns_refine, 2 n words per column and n d)
             p->rs_x0 = (int)sq32(K);
             // (+ K qcap + qcap: the moved block of refine_kept_columns)
-            p->rs_stride = (p->rs_x0 + 6 * K * p->qcap + p->qcap + 31) / 32 * 32;
+            p->rs_stride = ns ? (2ll * n * p->qcap + n * d + 31) / 32 * 32
+                              : (p->rs_x0 + 6 * K * p->qcap + p->qcap + 31) / 32 * 32;
             long long doubles = (long long)p->lp.grid * p->rs_stride;
             for (int c = 0; c < p->lp.n_fb; ++c) {
                 FallbackClass& f = p->lp.fb[c];
                 f.rs_x0 = (int)sq32(f.K);
-                f.rs_stride = (f.rs_x0 + 5 * f.K + 31) / 32 * 32;
+                f.rs_stride = ns ? ((2ll + d) * f.n + 31) / 32 * 32 : (f.rs_x0 + 5 * f.K + 31) / 32 * 32;
                 if ((long long)f.grid * f.rs_stride > doubles) doubles = (long long)f.grid * f.rs_stride;
             }
             p->rs_doubles = doubles;
@@ -668,11 +693,11 @@ int rbffd_assemble(rbffd_plan_t p, void* stream, rbffd_csr* out) {
     a.fb_flag = p->fb_flag; a.fb_list = p->fb_list;
     a.slot_w = p->slot_w; a.slot_lam = p->slot_lam; a.slot_pass = p->slot_pass; a.ctr = p->ctr;
     a.no_seed = p->opts.fault_inject == 1;
-    a.factor = p->opts.factor;
+    a.lay = p->lay;
     a.max_ctas = p->opts.max_ctas;
     a.elastic = p->opts.elastic;
     a.rs = p->rs;
-    a.fma_r2 = p->rs == nullptr ? 1 : 0;
+    a.fma_r2 = p->rs == nullptr ? 1 : 0;  // (saddle-point layouts)
     a.rs_stride = p->rs_stride;
     a.rs_x0 = p->rs_x0;
     a.refine_min_K = p->refine_min_K;

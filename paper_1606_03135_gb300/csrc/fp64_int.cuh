@@ -54,10 +54,15 @@ __device__ __forceinline__ double rcp_core(double x, bool* slow) {
     return __longlong_as_double((long long)(f == 0ull ? pb : nb));
 }
 
+// (out of line: the traversal kernels run several phases of different systems side by side, and
+// their instructions have to stay in the instruction caches)
+static __device__ __noinline__ double rcp_slow(double x) { return 1.0 / x; }
+static __device__ __noinline__ double sqrt_slow(double x) { return sqrt(x); }
+
 __device__ __forceinline__ double rcp_fixed(double x) {
     bool slow;
     const double r = rcp_core(x, &slow);
-    return slow ? 1.0 / x : r;
+    return slow ? rcp_slow(x) : r;
 }
 
 // Square root of an FP64 value with three FP64 instructions.  A 24-bit seed y0 of 1/sqrt(m)
@@ -69,7 +74,7 @@ __device__ __forceinline__ double rcp_fixed(double x) {
 __device__ __forceinline__ double sqrt_fast(double x) {
     const unsigned long long b = (unsigned long long)__double_as_longlong(x);
     const int e = (int)(b >> 52);  // the sign bit is included: negative x takes the slow path
-    if (e == 0 || e >= 0x7ff) return sqrt(x);
+    if (e == 0 || e >= 0x7ff) return sqrt_slow(x);
     const int k = e - 1023;  // x = m 2^k, m in [1, 2)
     const int odd = k & 1;
     const int h2 = (k - odd) >> 1;  // x = m' 4^h2 with m' = m or 2m in [1, 4)

@@ -80,6 +80,9 @@ int cuda_status(cudaError_t e, const char* what, int line);
 #define RB_CUDA(call) ::rbffd::cuda_status((call), #call, __LINE__)
 #define RB_LAUNCHED(what) ::rbffd::cuda_status(cudaGetLastError(), what, __LINE__)
 
+// start of row i of a packed lower triangle
+__host__ __device__ __forceinline__ int tri(int i) { return (i * (i + 1)) >> 1; }
+
 __device__ __forceinline__ void set_error(DevCounters* c, int code) {
     atomicCAS(&c->status, 0, code);
 }
@@ -155,7 +158,7 @@ struct SolveArgs {
                                    // position per node (nullptr: the stencil's center)
     double coef;               // m (m + D - 2)
     int no_seed;               // fault injection: push no initial center (waits run out)
-    int factor;                // RBFFD_FACTOR_LDLT (packed layout) or RBFFD_FACTOR_LU (full)
+    int lay;                   // layout of the local systems (kLay...)
     int max_ctas;              // cap on the persistent grid (0 = fill the GPU)
     int elastic;               // > 0: a CTA holding no queue slot leaves when this many wait
     int fma_r2;                // 1: squared distances of the local systems with FMA (plans
@@ -187,8 +190,14 @@ struct SolveArgs {
     DevCounters* ctr;
 };
 
-size_t solve_smem_per_cta(int n, int K, int qcap, int qmax, int D, int packed,
-                          int* stride_out);
+// Layout of the local systems of a plan: the full matrix (LU), the packed lower triangle
+// (LDL^T), or the null space of the polynomial constraints (nullspace.cuh).
+constexpr int kLayFull = 0, kLayPacked = 1, kLayNull = 2;
+
+size_t solve_smem_per_cta(int n, int K, int qcap, int qmax, int D, int lay, int* stride_out);
+// Kernels of nullspace.cu by team size (nullptr: no such team).
+const void* null_traversal_kernel(int D, int nt, bool chunked);
+const void* null_fallback_kernel(int D, int nt);
 size_t basis_smem_bytes(int count);
 
 // Launch geometry decided once per plan.  Fallback re-solves run per stencil class (one
@@ -210,7 +219,7 @@ struct LaunchPlan {
     int n_fb = 0;
     FallbackClass fb[kMaxEll + 1];
 };
-int prepare_solve_kernels(int D, int packed, int n, int K, int qcap, int qmax, int basis_count,
+int prepare_solve_kernels(int D, int lay, int n, int K, int qcap, int qmax, int basis_count,
                           LaunchPlan* lp);
 int launch_centroid_ref(int D, const double* X, const int* nbr, const int* node_n, int N, int ns,
                         unsigned char* ref_pos, cudaStream_t s, int* launches);

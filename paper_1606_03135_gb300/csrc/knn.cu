@@ -211,25 +211,25 @@ __device__ __forceinline__ int cell_index(const GridParams& g, const int* c) {
 
 template <int D>
 __global__ void k_cell_count(const double* __restrict__ X, int N, const GridParams* __restrict__ gp,
-                             int* __restrict__ cell_of, int* __restrict__ count) {
+                             int* __restrict__ cell_of, int* __restrict__ count,
+                             int* __restrict__ rank) {
     const GridParams g = *gp;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) {
         int c[3];
         for (int a = 0; a < D; ++a) c[a] = cell_coord<D>(g, X[(size_t)i * D + a], a);
         int id = cell_index<D>(g, c);
         cell_of[i] = id;
-        atomicAdd(&count[id], 1);
+        rank[i] = atomicAdd(&count[id], 1);
     }
 }
 
 template <int D>
 __global__ void k_cell_fill(const double* __restrict__ X, int N, const int* __restrict__ cell_of,
-                            const int* __restrict__ cell_start, int* __restrict__ cursor,
+                            const int* __restrict__ cell_start, const int* __restrict__ rank,
                             int* __restrict__ sorted_idx, double* __restrict__ sorted_X,
                             float* __restrict__ sorted_Xf) {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) {
-        int c = cell_of[i];
-        int pos = cell_start[c] + atomicAdd(&cursor[c], 1);
+        const int pos = cell_start[cell_of[i]] + rank[i];
         sorted_idx[pos] = i;
         for (int a = 0; a < D; ++a) {
             const double x = X[(size_t)i * D + a];
@@ -249,10 +249,9 @@ __device__ __forceinline__ bool key_less(unsigned long long ka, int ia, unsigned
 // the box can reach (+inf when the box covers the whole grid).  (The query's exact distance to
 // the box faces is larger, but admitting more candidates only makes the sort dearer.)
 template <int D>
-__device__ __forceinline__ bool ring_box(const GridParams& g, const double* xq, const int* c0,
-                                         int r, int* clo, int* chi, unsigned long long* bkey,
+__device__ __forceinline__ bool ring_box(const GridParams& g, const int* c0, int r,
+                                         int* clo, int* chi, unsigned long long* bkey,
                                          float* thr) {
-    (void)xq;
     bool all = true;
     for (int a = 0; a < D; ++a) {
         clo[a] = max(c0[a] - r, 0);
@@ -264,7 +263,8 @@ __device__ __forceinline__ bool ring_box(const GridParams& g, const double* xq, 
     *bkey = dkey(all ? __longlong_as_double(0x7ff0000000000000LL)  // +inf
                      : R2);
     // FP32 screen threshold (screen_outside): above R2 by more than the screen's rounding
-    *thr = all ? __int_as_float(0x7f800000) : __double2float_ru(R2 * (1.0 + 0x1p-19));
+    *thr = all ? __int_as_float(0x7f800000)
+               : __fmul_ru(__double2float_ru(R2), 1.0f + 0x1p-19f);
     return all;
 }
 
@@ -293,20 +293,22 @@ __device__ __forceinline__ bool screen_outside(const float* qf, const float* __r
 template <int D>
 __device__ __forceinline__ int first_ring(const GridParams& g, const int* c0, int n,
                                           const int* __restrict__ cell_start) {
-    int lo[3], hi[3];
+    int lo[3] = {0, 0, 0}, hi[3] = {0, 0, 0};
     for (int a = 0; a < D; ++a) {
         lo[a] = max(c0[a] - 1, 0);
         hi[a] = min(c0[a] + 1, g.dims[a] - 1);
     }
-    int cnt = 0, cells = 0;
-    const int nz = (D == 3) ? hi[2] - lo[2] + 1 : 1;
-    for (int rz = 0; rz < nz; ++rz)
-        for (int ry = lo[1]; ry <= hi[1]; ++ry) {
-            int cc[3] = {lo[0], ry, (D == 3) ? lo[2] + rz : 0};
-            const int row0 = cell_index<D>(g, cc);
-            cnt += cell_start[row0 + (hi[0] - lo[0]) + 1] - cell_start[row0];
-            cells += hi[0] - lo[0] + 1;
-        }
+    const int nx = hi[0] - lo[0] + 1, ny = hi[1] - lo[1] + 1, rows = ny * (hi[2] - lo[2] + 1);
+    const int lane = threadIdx.x & 31;
+    int cnt = 0;
+    if (lane < rows) {  // (at most 9: a lane per row)
+        const int rz = lane / ny;
+        const int cc[3] = {lo[0], lo[1] + lane - rz * ny, lo[2] + rz};
+        const int row0 = cell_index<D>(g, cc);
+        cnt = cell_start[row0 + nx] - cell_start[row0];
+    }
+    cnt = __reduce_add_sync(0xffffffffu, cnt);
+    const int cells = nx * rows;
     const float per = fmaxf((float)cnt / (float)cells, 0.05f);  // nodes per cell
     const float vol = (D == 2) ? 3.14159265f : 4.18879020f;
     const float rad = (D == 2) ? sqrtf((float)n / (per * vol)) : cbrtf((float)n / (per * vol));
@@ -329,7 +331,7 @@ __device__ int knn_stream(const GridParams& g, const double* xq, const float* xq
         int clo[3], chi[3];
         unsigned long long bkey;
         float thr;
-        const bool all = ring_box<D>(g, xq, c0, r, clo, chi, &bkey, &thr);
+        const bool all = ring_box<D>(g, c0, r, clo, chi, &bkey, &thr);
         cnt = 0;
         cur = 0;
         const int ny = chi[1] - clo[1] + 1;
@@ -397,13 +399,129 @@ __device__ int knn_stream(const GridParams& g, const double* xq, const float* xq
     return cur;
 }
 
+// In-lane pieces of warp_sort, ascending: R registers in any order (lane_sort) or holding a
+// bitonic sequence (lane_merge; R = 3 is sorted in full, larger R halve down to 1 or 3).
+__device__ __forceinline__ void order2(unsigned& a, unsigned& b) {
+    const unsigned t = min(a, b);
+    b = max(a, b);
+    a = t;
+}
+
+template <int R>
+__device__ __forceinline__ void lane_merge(unsigned* v) {
+    if constexpr (R == 3) {
+        order2(v[0], v[1]);
+        order2(v[1], v[2]);
+        order2(v[0], v[1]);
+    } else if constexpr (R > 1) {
+#pragma unroll
+        for (int r = 0; r < R / 2; ++r) order2(v[r], v[r + R / 2]);
+        lane_merge<R / 2>(v);
+        lane_merge<R / 2>(v + R / 2);
+    }
+}
+
+template <int R>
+__device__ __forceinline__ void lane_sort(unsigned* v) {
+    if constexpr (R == 3) {
+        lane_merge<3>(v);
+    } else if constexpr (R > 1) {
+        lane_sort<R / 2>(v);
+        lane_sort<R / 2>(v + R / 2);
+#pragma unroll
+        for (int r = 0; r < R / 2; ++r) order2(v[r], v[R - 1 - r]);
+        lane_merge<R / 2>(v);
+        lane_merge<R / 2>(v + R / 2);
+    }
+}
+
+// The order of a warp's cnt <= 32 R collected candidates by (key, index): ord[t] = the place of
+// the t-th.  A 32-bit word per candidate, its key's upper bits (a monotone map: 16 bits of
+// mantissa and the 128 binades below the largest key; smaller keys map to 0) above its place, is
+// sorted in registers: lane l holds elements l R .. l R + R - 1 of a bitonic network whose steps
+// across lanes are one shuffle and one min or max per word.  Candidates whose words share the
+// upper bits (equal distances, as on lattices, or nearly equal ones) are then put in the exact
+// order by exchanging neighbours until none is out of order.
+// Bound by issue slots: the network on 64-bit keys and indices in shared memory that this
+// replaced took about 22 slots and two shared-memory round trips per pair and step, this one 3 (with
+// the rows' lookup by masks below, a stencil call of 20,000 nodes in 3D, n = 45: 240 -> 135 us).
+template <int R>
+__device__ __forceinline__ void warp_sort(const unsigned long long* wk, const int* wi, int cnt,
+                                          unsigned short* ord) {
+    const int lane = threadIdx.x & 31;
+    unsigned v[R], top = 0;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int e = lane + 32 * r;
+        v[r] = e < cnt ? (unsigned)(wk[e] >> 32) : 0u;
+        top = max(top, v[r]);
+    }
+    top = __reduce_max_sync(0xffffffffu, top);  // (< 2^31)
+    const unsigned base = max(top + 1u, 1u << 27) - (1u << 27);
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int e = lane + 32 * r;
+        const unsigned q = max(v[r], base) - base;  // < 2^27
+        v[r] = e < cnt ? ((q >> 4) << 9) | (unsigned)e : ~0u;
+    }
+    lane_sort<R>(v);
+#pragma unroll 1
+    for (int k = 2; k <= 32; k <<= 1) {  // merge the sorted runs of k/2 lanes
+        unsigned t[R];
+        bool low = (lane & (k >> 1)) == 0;
+#pragma unroll
+        for (int r = 0; r < R; ++r) t[r] = __shfl_xor_sync(0xffffffffu, v[R - 1 - r], k - 1);
+#pragma unroll
+        for (int r = 0; r < R; ++r) v[r] = low ? min(v[r], t[r]) : max(v[r], t[r]);
+#pragma unroll 1
+        for (int j = k >> 2; j > 0; j >>= 1) {
+            low = (lane & j) == 0;
+#pragma unroll
+            for (int r = 0; r < R; ++r) t[r] = __shfl_xor_sync(0xffffffffu, v[r], j);
+#pragma unroll
+            for (int r = 0; r < R; ++r) v[r] = low ? min(v[r], t[r]) : max(v[r], t[r]);
+        }
+        lane_merge<R>(v);
+    }
+    const unsigned after = __shfl_down_sync(0xffffffffu, v[0], 1);  // (lane 31: its own)
+    bool tie = lane < 31 && after != ~0u && (after >> 9) == (v[R - 1] >> 9);
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        ord[lane * R + r] = (unsigned short)(v[r] & 511u);
+        if (r + 1 < R) tie = tie || (v[r + 1] != ~0u && (v[r + 1] >> 9) == (v[r] >> 9));
+    }
+    __syncwarp();
+    if (!__any_sync(0xffffffffu, tie)) return;
+    for (;;) {
+        bool swapped = false;
+#pragma unroll 1
+        for (int phase = 0; phase < 2; ++phase) {
+            for (int i = 2 * lane + phase; i + 1 < cnt; i += 64) {
+                const int a = ord[i], b = ord[i + 1];
+                if (key_less(wk[b], wi[b], wk[a], wi[a])) {
+                    ord[i] = (unsigned short)b;
+                    ord[i + 1] = (unsigned short)a;
+                    swapped = true;
+                }
+            }
+            __syncwarp();
+        }
+        if (!__any_sync(0xffffffffu, swapped)) return;
+    }
+}
+
 // One warp per query node.  Usual case: every candidate of the search box that lies inside
 // the guaranteed radius is collected into shared memory (growing the ring until there are n),
-// and the warp sorts them by (IEEE bits of d2, index) with a bitonic network; the first n
-// are the stencil.  Boxes with more such candidates than the buffer holds (256, or 512 for
+// and the warp sorts them by (IEEE bits of d2, index) (warp_sort); the first n are the stencil.  Boxes with more such candidates than the buffer holds (256, or 512 for
 // stencils of more than 64 nodes) take the streaming search instead.  Either way the order is
 // exact.
 __host__ __device__ __forceinline__ int knn_collect_cap(int n) { return n > 64 ? 512 : 256; }
+
+// Ints of a warp's scratch: the rows' table (64) and the FP32 screen's queue (64), and, once the
+// candidates are collected, their order (16 bits each).
+__host__ __device__ __forceinline__ int knn_ints(int n) {
+    return max(128, knn_collect_cap(n) / 2);
+}
 
 __host__ __device__ __forceinline__ int knn_words(int n) {  // per-warp buffer entries
     return max(2 * n + 32, knn_collect_cap(n));
@@ -412,6 +530,7 @@ __host__ __device__ __forceinline__ int knn_words(int n) {  // per-warp buffer e
 template <int D>
 __global__ void __launch_bounds__(256) k_knn(const double* __restrict__ X, int N, int n,
                                              double omd2, const GridParams* __restrict__ gp,
+                                             const int* __restrict__ cell_of,
                                              const int* __restrict__ cell_start,
                                              const int* __restrict__ sorted_idx,
                                              const double* __restrict__ sorted_X,
@@ -426,9 +545,8 @@ __global__ void __launch_bounds__(256) k_knn(const double* __restrict__ X, int N
     const int W = knn_words(n);
     unsigned long long* wk = knn_smem + (size_t)wib * W;
     int* wi = reinterpret_cast<int*>(knn_smem + (size_t)wpb * W) + (size_t)wib * W;
-    int* soff = reinterpret_cast<int*>(knn_smem + (size_t)wpb * W) + (size_t)wpb * W + wib * 128;
-    int* sbeg = soff + 32;
-    int* squeue = soff + 64;  // candidates that passed the FP32 screen, awaiting FP64 (< 64)
+    int* srow = reinterpret_cast<int*>(knn_smem + (size_t)wpb * W) + (size_t)wpb * W + wib * knn_ints(n);
+    int* squeue = srow + 64;  // candidates that passed the FP32 screen, awaiting FP64 (< 64)
     const GridParams g = *gp;
 
     for (int q = blockIdx.x * wpb + wib; q < N; q += gridDim.x * wpb) {
@@ -438,7 +556,15 @@ __global__ void __launch_bounds__(256) k_knn(const double* __restrict__ X, int N
         for (int a = 0; a < D; ++a) {
             xq[a] = X[(size_t)q * D + a];
             xqf[a] = __double2float_rn(xq[a]);
-            c0[a] = cell_coord<D>(g, xq[a], a);
+        }
+        {  // the query's cell, as the counting pass found it
+            int c = cell_of[q];
+            for (int a = 0; a < D - 1; ++a) {
+                const int up = c / g.dims[a];
+                c0[a] = c - up * g.dims[a];
+                c = up;
+            }
+            c0[D - 1] = c;
         }
         const int kCollect = knn_collect_cap(n);
         // node q's own stencil size (per-node plans search only that many; row q of nbr is
@@ -450,15 +576,17 @@ __global__ void __launch_bounds__(256) k_knn(const double* __restrict__ X, int N
             int clo[3], chi[3];
             unsigned long long bkey;
             float thr;
-            all = ring_box<D>(g, xq, c0, r, clo, chi, &bkey, &thr);
+            all = ring_box<D>(g, c0, r, clo, chi, &bkey, &thr);
             cnt = 0;
             const int ny = chi[1] - clo[1] + 1;
             const int nz = (D == 3) ? chi[2] - clo[2] + 1 : 1;
             const int nrows = ny * nz;
             // The box's cell rows (contiguous ranges of the cell-sorted nodes) are packed into
             // full batches of 32 candidates: an FP64 warp instruction costs the same with idle
-            // lanes, and a row holds only a few nodes.  Lane l takes row g0 + l, the rows'
-            // offsets are scanned, and each candidate finds its row by binary search.
+            // lanes, and a row holds only a few nodes.  Lane l takes row g0 + l and the rows'
+            // offsets are scanned.  A batch's candidates find their rows by counting the rows
+            // that start at or before them: the non-empty rows' (first node - offset) are
+            // listed in order, and the starts inside the batch make a bit mask.
             for (int g0 = 0; g0 < nrows && cnt <= kCollect; g0 += 32) {
                 const int R = g0 + lane;
                 int beg = 0, len = 0;
@@ -475,8 +603,9 @@ __global__ void __launch_bounds__(256) k_knn(const double* __restrict__ X, int N
                     if (lane >= o) incl += t;
                 }
                 const int total = __shfl_sync(0xffffffffu, incl, 31);
-                soff[lane] = incl - len;
-                sbeg[lane] = beg;
+                const int off = incl - len;
+                const unsigned rows = __ballot_sync(0xffffffffu, len > 0);
+                if (len > 0) srow[__popc(rows & ((1u << lane) - 1u))] = beg - off;
                 __syncwarp();
                 // Each batch's candidates pass an FP32 screen first (screen_outside); those that
                 // may lie inside the guaranteed radius queue up, and their exact FP64 distances
@@ -487,14 +616,12 @@ __global__ void __launch_bounds__(256) k_knn(const double* __restrict__ X, int N
                     const int e = b0 + lane;
                     bool pass = false;
                     int p = 0;
+                    const bool starts = len > 0 && (unsigned)(off - b0) < 32u;
+                    const unsigned here =
+                        __reduce_or_sync(0xffffffffu, starts ? 1u << (off - b0) : 0u);
+                    const unsigned before = __ballot_sync(0xffffffffu, len > 0 && off < b0);
                     if (e < total) {
-                        int lo = 0, hi = 31;  // the last row whose offset is <= e (non-empty)
-                        while (lo < hi) {
-                            const int mid = (lo + hi + 1) >> 1;
-                            if (soff[mid] <= e) lo = mid;
-                            else hi = mid - 1;
-                        }
-                        p = sbeg[lo] + (e - soff[lo]);
+                        p = srow[__popc(before) + __popc(here & (~0u >> (31 - lane))) - 1] + e;
                         pass = !screen_outside<D>(xqf, sorted_Xf + (size_t)p * D, g.xerr, thr);
                     }
                     const unsigned pb = __ballot_sync(0xffffffffu, pass);
@@ -527,13 +654,14 @@ __global__ void __launch_bounds__(256) k_knn(const double* __restrict__ X, int N
                         qn = rest;
                     }
                 }
-                __syncwarp();  // soff/sbeg are rewritten by the next group
+                __syncwarp();  // srow is rewritten by the next group
             }
             if (cnt > kCollect || cnt >= nq || all) break;
             ++r;
         }
         const unsigned long long* rk;
         const int* ri;
+        const unsigned short* ord = nullptr;  // the entries' places in rk, ri (null: in order)
         if (cnt > kCollect) {  // too many candidates to sort: stream them
             __syncwarp();
             const int cur = knn_stream<D>(g, xq, xqf, c0, r, nq, cell_start, sorted_idx, sorted_X,
@@ -541,39 +669,30 @@ __global__ void __launch_bounds__(256) k_knn(const double* __restrict__ X, int N
             rk = wk + cur * nq;
             ri = wi + cur * nq;
         } else {
-            int P = 32;
-            while (P < cnt) P <<= 1;
-            for (int e = cnt + lane; e < P; e += 32) { wk[e] = ~0ull; wi[e] = 0x7fffffff; }
-            __syncwarp();
-            for (int k = 2; k <= P; k <<= 1)  // bitonic sort, ascending
-                for (int j = k >> 1; j > 0; j >>= 1) {
-                    const int lj = 31 - __clz(j);
-                    for (int t = lane; t < (P >> 1); t += 32) {
-                        const int i = ((t >> lj) << (lj + 1)) | (t & (j - 1));
-                        const int l = i + j;
-                        const unsigned long long ki = wk[i], kl = wk[l];
-                        const int ii = wi[i], il = wi[l];
-                        const bool up = (i & k) == 0;
-                        if (up ? key_less(kl, il, ki, ii) : key_less(ki, ii, kl, il)) {
-                            wk[i] = kl; wi[i] = il;
-                            wk[l] = ki; wi[l] = ii;
-                        }
-                    }
-                    __syncwarp();
-                }
+            // (the rows' table and the queue are free now)
+            unsigned short* o = reinterpret_cast<unsigned short*>(srow);
+            if (cnt <= 32) warp_sort<1>(wk, wi, cnt, o);
+            else if (cnt <= 64) warp_sort<2>(wk, wi, cnt, o);
+            else if (cnt <= 96) warp_sort<3>(wk, wi, cnt, o);
+            else if (cnt <= 128) warp_sort<4>(wk, wi, cnt, o);
+            else if (cnt <= 192) warp_sort<6>(wk, wi, cnt, o);
+            else if (cnt <= 256) warp_sort<8>(wk, wi, cnt, o);
+            else warp_sort<16>(wk, wi, cnt, o);
+            ord = o;
             rk = wk;
             ri = wi;
         }
         // write the stencil (the nq nearest), its width and retention ball
-        const double r2k = __longlong_as_double((long long)rk[nq - 1]);
+        const double r2k = __longlong_as_double((long long)rk[ord ? ord[nq - 1] : nq - 1]);
         const double rball = __dmul_rn(omd2, r2k);
         int blen = 0;
         for (int t0 = 0; t0 < n; t0 += 32) {
             const int t = t0 + lane;
             bool inb = false;
             if (t < nq) {
-                const int id = ri[t];
-                const double dd = __longlong_as_double((long long)rk[t]);
+                const int at = ord ? ord[t] : t;
+                const int id = ri[at];
+                const double dd = __longlong_as_double((long long)rk[at]);
                 nbr[(size_t)q * n + t] = id;
                 inb = dd <= rball;
                 if (t >= 1 && dd == 0.0) set_error(ctr, RBFFD_EDUPLICATE);
@@ -583,13 +702,13 @@ __global__ void __launch_bounds__(256) k_knn(const double* __restrict__ X, int N
             blen += __popc(__ballot_sync(0xffffffffu, inb));
         }
         if (lane == 0) {
-            if (ri[0] != q) set_error(ctr, RBFFD_EDUPLICATE);
+            if (ri[ord ? ord[0] : 0] != q) set_error(ctr, RBFFD_EDUPLICATE);
             rho2[q] = r2k;
             ball_len[q] = blen;
             atomicMax(&ctr->max_ball, blen);
         }
         for (int t = 1 + lane; t < blen; t += 32) {
-            const int i = ri[t];
+            const int i = ri[ord ? ord[t] : t];
             if (i > q) atomicAdd(&indeg[i], 1);
         }
         __syncwarp();
@@ -644,7 +763,7 @@ static size_t round256(size_t b) { return (b + 255) & ~size_t(255); }
 
 size_t grid_scratch_bytes(int N, int D, int ncell_max) {
     size_t b = round256(sizeof(GridParams)) + round256(sizeof(BBoxAcc));
-    b += 3 * round256((size_t)(ncell_max + 1) * sizeof(int));  // count, start, cursor
+    b += 3 * round256((size_t)(ncell_max + 1) * sizeof(int));  // count, start, one to spare
     b += 2 * round256((size_t)N * sizeof(int));                // cell_of, sorted_idx
     b += round256((size_t)N * D * sizeof(double));             // sorted_X
     b += round256((size_t)N * D * sizeof(float));              // sorted_Xf (FP32 screen)
@@ -664,17 +783,16 @@ static int grid_and_knn(const double* X, int N, int n, double omd2, void* scratc
     GridParams* gp = reinterpret_cast<GridParams*>(take(sizeof(GridParams)));
     BBoxAcc* acc = reinterpret_cast<BBoxAcc*>(take(sizeof(BBoxAcc)));
     int* count = reinterpret_cast<int*>(take((size_t)(ncell_max + 1) * sizeof(int)));
+    const size_t zeros = p - reinterpret_cast<char*>(acc);  // (acc and count, side by side)
     int* start = reinterpret_cast<int*>(take((size_t)(ncell_max + 1) * sizeof(int)));
-    int* cursor = reinterpret_cast<int*>(take((size_t)(ncell_max + 1) * sizeof(int)));
+    int* rank = ball_len;  // a node's place in its cell, until k_knn writes the ball lengths
     int* cell_of = reinterpret_cast<int*>(take((size_t)N * sizeof(int)));
     int* sorted_idx = reinterpret_cast<int*>(take((size_t)N * sizeof(int)));
     double* sorted_X = reinterpret_cast<double*>(take((size_t)N * D * sizeof(double)));
     float* sorted_Xf = reinterpret_cast<float*>(take((size_t)N * D * sizeof(float)));
 
     int rc;
-    if ((rc = RB_CUDA(cudaMemsetAsync(acc, 0, sizeof(BBoxAcc), s))) ||
-        (rc = RB_CUDA(cudaMemsetAsync(count, 0, (size_t)(ncell_max + 1) * sizeof(int), s))) ||
-        (rc = RB_CUDA(cudaMemsetAsync(cursor, 0, (size_t)(ncell_max + 1) * sizeof(int), s))) ||
+    if ((rc = RB_CUDA(cudaMemsetAsync(acc, 0, zeros, s))) ||
         (rc = RB_CUDA(cudaMemsetAsync(indeg, 0, (size_t)N * sizeof(int), s))))
         return rc;
     const int tb = 256;
@@ -683,20 +801,20 @@ static int grid_and_knn(const double* X, int N, int n, double omd2, void* scratc
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     k_grid_params<D><<<nb < sms ? nb : sms, tb, 0, s>>>(X, N, n, ncell_max, acc, gp);
-    k_cell_count<D><<<nb, tb, 0, s>>>(X, N, gp, cell_of, count);
+    k_cell_count<D><<<nb, tb, 0, s>>>(X, N, gp, cell_of, count, rank);
     k_scan<int, int><<<1, 1024, 0, s>>>(count, start, ncell_max, &gp->ncell);
-    k_cell_fill<D><<<nb, tb, 0, s>>>(X, N, cell_of, start, cursor, sorted_idx, sorted_X,
+    k_cell_fill<D><<<nb, tb, 0, s>>>(X, N, cell_of, start, rank, sorted_idx, sorted_X,
                                      sorted_Xf);
     const int wpb = 8;
     const int words = knn_words(n);
-    size_t smem = (size_t)wpb * (words * (sizeof(unsigned long long) + sizeof(int)) + 128 * sizeof(int));
+    size_t smem = (size_t)wpb * (words * (sizeof(unsigned long long) + sizeof(int)) + knn_ints(n) * sizeof(int));
     if (smem > 48 * 1024 &&
         (rc = RB_CUDA(cudaFuncSetAttribute(k_knn<D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            (int)smem))))
         return rc;
     int blocks = (N + wpb - 1) / wpb;
-    k_knn<D><<<blocks, wpb * 32, smem, s>>>(X, N, n, omd2, gp, start, sorted_idx, sorted_X,
-                                            sorted_Xf, nbr, rho2, ball_len, indeg, node_n, ctr);
+    k_knn<D><<<blocks, wpb * 32, smem, s>>>(X, N, n, omd2, gp, cell_of, start, sorted_idx,
+                                            sorted_X, sorted_Xf, nbr, rho2, ball_len, indeg, node_n, ctr);
     *launches += 5;
     return RB_LAUNCHED(__func__);
 }

@@ -1532,7 +1532,7 @@ __device__ __forceinline__ int ns_refine_log2(int M) { return M > 40 ? 7 : 10; }
 
 template <int D, int NT>
 __device__ __noinline__ void ns_refine(const SolveArgs& a, const Shape& sh, int j, int c0, int qk,
-                                       const NullSmem& sm, int kind, double* __restrict__ gw) {
+                                       const NullSmem& sm, int kind, double* gw) {
     const int tid = threadIdx.x, lane = tid & 31, n = sh.n, M = sh.M, s = n - M, m = sh.m;
     const int eB = s_ns_eb;
     double *gW = gw, *gR = gw + (size_t)n * qk, *gX = gw + (size_t)2 * n * qk;
@@ -1551,55 +1551,62 @@ __device__ __noinline__ void ns_refine(const SolveArgs& a, const Shape& sh, int 
         gW[e] = p < M ? sm.T[(n + c0 + c) * sm.ldm + p] : sm.X[c * sm.ldx + sm.x2 + p - M];
     }
     __syncthreads();
-    // rho: four columns per thread share the entries of A
-    const int groups = (qk + 3) >> 2;
+    // rho: four columns share the entries of A, four lanes a row (a quarter of its terms each, summed
+    // in one order whatever the team; with a lane per row 113 of a team's 256 threads walked 113
+    // dependent terms: 3D degree 5, N = 4,000, delta = 1 6.93 ms of traversal, now 6.67)
+    const int groups = (qk + 3) >> 2, part = (n + 3) >> 2, l4 = lane & 3;
 #pragma unroll 1
-    for (int e = tid; e < n * groups; e += NT) {
-        const int g = small_div(e, n), p = e - g * n, nc = min(4, qk - 4 * g);
+    for (int e = tid; e < ((4 * n * groups + 31) & ~31); e += NT) {  // (whole warps)
+        const int item = min(e >> 2, n * groups - 1);
+        const int g = small_div(item, n), p = item - g * n, nc = min(4, qk - 4 * g);
         double x[D], r[4] = {};
-        for (int d = 0; d < D; ++d) x[d] = __ldcg(&gX[p * D + d]);
+        for (int d = 0; d < D; ++d) x[d] = gX[p * D + d];
         const double* w = gW + (size_t)4 * g * n;
-#pragma unroll 1
-        for (int v = 0; v < n; ++v) {
-            if (v == p) continue;
+        const int v1 = min((l4 + 1) * part, n);
+#pragma unroll 2
+        for (int v = l4 * part; v < v1; ++v) {
             double y[D];
-            for (int d = 0; d < D; ++d) y[d] = __ldcg(&gX[v * D + d]);
-            const double r2 = sqdist_rn<D>(x, y);
+            for (int d = 0; d < D; ++d) y[d] = gX[v * D + d];
+            const double r2 = v == p ? 1.0 : sqdist_rn<D>(x, y);
             double pm = sqrt_fast(r2);
 #pragma unroll 1
             for (int k = 0; k < (m - 1) / 2; ++k) pm = __dmul_rn(pm, r2);
+            if (v == p) pm = 0.0;
 #pragma unroll
             for (int c = 0; c < 4; ++c)
-                if (c < nc) r[c] = fma(-pm, __ldcg(&w[c * n + v]), r[c]);
+                if (c < nc) r[c] = fma(-pm, w[c * n + v], r[c]);
         }
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
-            if (c >= nc) continue;
-            double f = 0.0;
-            if (kind == 2) {
-                f = neumann_at<D>(a, sh, j, 0, x);
-            } else if (sm.order[p] != sm.cols[c0 + 4 * g + c]) {
-                double y[D];
-                const int t = sm.pos[sm.cols[c0 + 4 * g + c]];
-                for (int d = 0; d < D; ++d) y[d] = __ldcg(&gX[t * D + d]);
-                const double r2 = sqdist_rn<D>(x, y);
-                double pm2 = sqrt_fast(r2);
-#pragma unroll 1
-                for (int k = 0; k < (m - 3) / 2; ++k) pm2 = __dmul_rn(pm2, r2);
-                f = __dmul_rn(sh.coef, pm2);
-            }
-            gR[(4 * g + c) * n + p] = f + r[c];
+            r[c] += __shfl_xor_sync(0xffffffffu, r[c], 1);
+            r[c] += __shfl_xor_sync(0xffffffffu, r[c], 2);
         }
+        if (l4 >= nc || e >= 4 * n * groups) continue;
+        const int c = 4 * g + l4;  // lane l4 adds f of the group's column l4
+        double f = l4 == 0 ? r[0] : (l4 == 1 ? r[1] : (l4 == 2 ? r[2] : r[3]));
+        if (kind == 2) {
+            f += neumann_at<D>(a, sh, j, 0, x);
+        } else if (sm.order[p] != sm.cols[c0 + c]) {
+            double y[D];
+            const int t = sm.pos[sm.cols[c0 + c]];
+            for (int d = 0; d < D; ++d) y[d] = gX[t * D + d];
+            const double r2 = sqdist_rn<D>(x, y);
+            double pm2 = sqrt_fast(r2);
+#pragma unroll 1
+            for (int k = 0; k < (m - 3) / 2; ++k) pm2 = __dmul_rn(pm2, r2);
+            f += __dmul_rn(sh.coef, pm2);
+        }
+        gR[c * n + p] = f;
     }
     __syncthreads();
 #pragma unroll 1
     for (int c = tid >> 5; c < qk; c += NT / 32) {  // rho_basic to limbs, in the words of f1
         int e = -200;
 #pragma unroll 1
-        for (int p = lane; p < M; p += 32) e = max(e, scale_exp(__ldcg(&gR[c * n + p])));
+        for (int p = lane; p < M; p += 32) e = max(e, scale_exp(gR[c * n + p]));
         e = __reduce_max_sync(0xffffffffu, e);
 #pragma unroll 1
-        for (int p = lane; p < M; p += 32) limbs(sm.X + c * sm.ldx)[p] = to_limbs(__ldcg(&gR[c * n + p]), e);
+        for (int p = lane; p < M; p += 32) limbs(sm.X + c * sm.ldx)[p] = to_limbs(gR[c * n + p], e);
         if (lane == 0) sm.ev[c] = (short)e;
     }
     __syncthreads();
@@ -1613,7 +1620,7 @@ __device__ __noinline__ void ns_refine(const SolveArgs& a, const Shape& sh, int 
             if ((k & 15) == 15) t.fold();
         }
         sm.X[c * sm.ldx + sm.x2 + i] =
-            __ldcg(&gR[c * n + M + i]) - from_fixed(t.total(), eB + sm.ev[c] + kSumUnit);
+            gR[c * n + M + i] - from_fixed(t.total(), eB + sm.ev[c] + kSumUnit);
     }
     __syncthreads();
     ns_forward<NT>(s, qk, sm);
@@ -1623,7 +1630,7 @@ __device__ __noinline__ void ns_refine(const SolveArgs& a, const Shape& sh, int 
 #pragma unroll 1
     for (int e = tid; e < s * qk; e += NT) {
         const int c = small_div(e, s), i = e - c * s;
-        sm.X[c * sm.ldx + sm.x2 + i] += __ldcg(&gW[c * n + M + i]);
+        sm.X[c * sm.ldx + sm.x2 + i] += gW[c * n + M + i];
     }
     if (tid == 0) atomicAdd(&a.ctr->sum_k2r, (unsigned long long)sh.K * sh.K * qk);
     __syncthreads();

@@ -519,16 +519,14 @@ int plan_impl(const double* nodes, int64_t N, int d, int n, int ell, int m,
         // Layouts to try.  LDL^T solves systems of one shape in the null space of the constraints
         // when r^m is conditionally definite there (ell >= (m - 1) / 2) and the fixed-point forms
         // are as accurate as the saddle-point factorization against a double-double solve: up to
-        // r^7 and degree 4 the norms of their errors are 0.3 to 1.0 times its over a set's rows.
-        // At degree 5 one-sided stencils are several times further off unless refined, as systems
-        // of K >= 100 are (2.6e-11 against the refined saddle-point solve's 2.6e-11); at degree 6
-        // and above (the constraints' pivots get small) and at r^9 and above (r^m spans more of the
-        // 58 bits) all are.  Refined systems with n > 3 M are left out as well: S is nearly the
-        // whole matrix there (n = 128, M = 21: 5.0 ms against 5.35).  Those, plans of several shapes
-        // and systems too large for this layout factor the saddle-point matrix.
-        const bool large = p->K >= RBFFD_REFINE_MIN_K;
-        const bool null_space = ldlt && one_shape && 2 * ell + 1 >= m && m <= 7 &&
-                                (large ? ell <= 5 && n <= 3 * (p->K - n) : ell <= 4);
+        // r^7 and degree 5 the norms of their errors over a set's rows are 0.5 to 1.0 times its
+        // (1.3 on a set whose largest error is one row's).  At degree 6 and above (the constraints'
+        // pivots get small) and at r^9 and above (r^m spans more of the 58 bits) they are larger.
+        // Large systems (K >= 100, which refine) with n > 3 M are left out as well: S is nearly the
+        // whole matrix there (n = 128, M = 21: 5.0 ms against 5.35).  Those, plans of several
+        // shapes and systems too large for this layout factor the saddle-point matrix.
+        const bool null_space = ldlt && one_shape && 2 * ell + 1 >= m && m <= 7 && ell <= 5 &&
+                                (p->K < RBFFD_REFINE_MIN_K || n <= 3 * (p->K - n));
         const int qcap0 = p->qcap;
         for (p->lay = null_space ? kLayNull : (ldlt ? kLayPacked : kLayFull);; p->lay = kLayPacked) {
             for (p->qcap = qcap0;; --p->qcap) {

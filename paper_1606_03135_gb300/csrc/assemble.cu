@@ -16,7 +16,7 @@
 // Local solve (one team of 32 to 512 threads per stencil).  The (n+M) x (n+M) saddle-point
 // matrix [A P; P^T 0] of §4.1 and the q right-hand sides of the overlapped system (one per
 // solved ball member) are formed in shared memory.  Plans whose stencils have one shape with
-// degree up to 4 (5 for K >= 100) and r^7 or below solve in the null space of P^T
+// degree up to 5 and r^7 or below solve in the null space of P^T
 // (nullspace.cuh: most of the work in fixed point on the integer pipe).  For the others the
 // lower triangle is stored packed and factored as L D L^T with Bunch-Kaufman pivoting, the
 // right-hand sides carried along ((1/3) K^3 + 2 K^2 q flops); the paper's

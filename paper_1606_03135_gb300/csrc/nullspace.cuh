@@ -17,7 +17,8 @@
 // (measured: 2.0 and 62.6).  In this form two thirds of the work are the two matrix products,
 // which run on the integer pipe in fixed point: operands are 59-bit integers in two limbs
 // (v = hi 2^28 + lo, |lo| <= 2^27) scaled by a power of two per matrix, a product is three
-// multiply-adds (hi hi, hi lo + lo hi; lo lo is below 2^-62 of the scale) and the sums are exact,
+// multiply-adds (hi hi, hi lo + lo hi; lo lo, below 2^-62 of the scale, only where S is formed) and
+// the sums are exact,
 // so the cancellation of S (entries near 0.1 out of sums near 100) costs nothing.
 #pragma once
 
@@ -29,6 +30,7 @@ namespace rbffd {
 // ------------------------------------------------------------------ fixed point
 constexpr int kFixBits = 58;   // |v| < 2^58 for an operand below its scale 2^e: v = x 2^(58 - e)
 constexpr int kLimbBits = 28;
+constexpr int kPowerBits = 62;  // of the powers of r and of f, which are not operands of products
 
 // The conversions and dot products below that are used in several places are functions of their
 // own, loops are not unrolled beyond what hides their latency, and quotients of small integers take
@@ -140,12 +142,37 @@ struct LimbSum {
         return h + ((m + (1ll << (kLimbBits - 1))) >> kLimbBits);
     }
 };
+
+// The same with the products of the lower limbs, for the sums that S is formed of: without them
+// (0.1 units a term) its weights of one-sided degree-5 stencils are 2 to 20 times further off.
+struct FullSum : LimbSum {
+    long long l = 0;
+    __device__ __forceinline__ void mac(int2 x, int2 y) {
+        LimbSum::mac(x, y);
+        l += (long long)x.y * y.y;
+    }
+    __device__ __forceinline__ void fold() {
+        m += l >> kLimbBits;
+        l &= (1ll << kLimbBits) - 1;
+        LimbSum::fold();
+    }
+    __device__ __forceinline__ long long total() const {
+        return h + ((m + (l >> kLimbBits) + (1ll << (kLimbBits - 1))) >> kLimbBits);
+    }
+};
 constexpr int kSumUnit = 2 * kLimbBits - 2 * kFixBits;  // -60
 
 // ------------------------------------------------------------------ shared-memory layout
 // Row stride of the tableau and of C in 8-byte words: an odd multiple of 16 bytes, so 16-byte
-// loads of consecutive rows hit distinct banks.
-__host__ __device__ __forceinline__ int ns_ldm(int M) { return 2 * (((M + 1) / 2) | 1); }
+// loads of consecutive rows hit distinct banks.  Systems of one column run in teams of one warp,
+// for which more of them per SM count for more than a two-way conflict, so there the pad is left
+// out (3D, M = 20, n = 45, N = 100k, delta = 1: 16 systems per SM instead of 14, 9.2 -> 8.7 ms;
+// with it left out at delta 0.4 and 0.2 too, 128-thread teams took 2% longer) unless rows would
+// then share a quarter of the banks (2D, M = 15: 1.60 -> 1.90 ms).
+__host__ __device__ __forceinline__ int ns_ldm(int M, int qmax) {
+    const int e = (M + 1) / 2;
+    return 2 * (qmax > 1 || (e & 3) == 0 ? e | 1 : e);
+}
 // A column's row of X: ns_x2 words (M of them and a pad for odd M, or s), then s more.
 __host__ __device__ __forceinline__ int ns_x2(int n, int M) {
     const int s = n - M, Mp = (M + 1) & ~1;
@@ -186,14 +213,15 @@ struct NullSmem {
 // S takes A11's place once C is formed, unless later chunks of columns need A11 (or it is larger).
 __host__ __device__ __forceinline__ bool ns_s_over_a11(int n, int M, int qcap, int qmax) {
     const int s = n - M;
-    return qcap >= qmax && s * (s + 1) / 2 <= M * ns_ldm(M);
+    return qcap >= qmax && s * (s + 1) / 2 <= M * ns_ldm(M, qmax);
 }
 
 // Bytes of one CTA's local system in this layout.
 __host__ __device__ __forceinline__ size_t ns_smem_bytes(int n, int M, int qcap, int qmax, int D) {
-    const size_t s = n - M, ldm = ns_ldm(M);
+    const size_t s = n - M, ldm = ns_ldm(M, qmax);
     const size_t tri_words = ns_s_over_a11(n, M, qcap, qmax) ? 0 : s * (s + 1) / 2;
-    const size_t words = (n + qmax + s) * ldm + qcap * (size_t)ns_ldx(n, M) + tri_words + n * D + 2 * s + qmax;
+    const size_t words = (n + qmax + s) * ldm + qcap * (size_t)ns_ldx(n, M) + tri_words + n * D +
+                         (qcap < qmax ? 2 * s : 0) + qmax;
     const size_t b = words * 8 + ((size_t)qmax + qcap) * 2 + 3 * (size_t)n + 2 * qmax;
     return (b + 15) & ~size_t(15);
 }
@@ -201,7 +229,7 @@ __host__ __device__ __forceinline__ size_t ns_smem_bytes(int n, int M, int qcap,
 template <int D>
 __device__ __forceinline__ void carve_ns(char* p, int n, int M, int qcap, int qmax, NullSmem& sm) {
     const int s = n - M;
-    sm.ldm = ns_ldm(M);
+    sm.ldm = ns_ldm(M, qmax);
     sm.ldx = ns_ldx(n, M);
     sm.x2 = ns_x2(n, M);
     double* w = reinterpret_cast<double*>(p);
@@ -217,11 +245,13 @@ __device__ __forceinline__ void carve_ns(char* p, int n, int M, int qcap, int qm
         w += s * (s + 1) >> 1;
     }
     sm.xi = w;
+    sm.rd = w;  // (the coordinates are done with when S is factored, unless later chunks need them)
     w += n * D;
-    sm.rd = w;
-    w += s;
-    sm.wb = w;
-    w += s;
+    if (qcap < qmax) {
+        sm.rd = w;
+        w += 2 * s;
+    }
+    sm.wb = sm.rd + s;
     sm.lam = w;
     w += qmax;
     short* h = reinterpret_cast<short*>(w);
@@ -552,37 +582,35 @@ __device__ void ns_product_c(int n, int M, int i0, int c0, int qk, int eA, const
 #pragma unroll 1
     for (int e = threadIdx.x; e < nr * nc; e += NT) {
         const int tr = small_div(e, nc), j = 2 * (e - tr * nc);
-        const int ia = i0 + 2 * tr, ib = min(ia + 1, rows - 1);
-        auto brow = [&](int i) { return sm.T + (i < s ? M + i : n + c0 + (i - s)) * ldm; };
-        const int4* pa = reinterpret_cast<const int4*>(brow(ia));
-        const int4* pb = reinterpret_cast<const int4*>(brow(ib));
-        const int4* pc = reinterpret_cast<const int4*>(sm.T + j);
-        const int lc = ldm >> 1;
-        LimbSum a0, a1, b0, b1;
+        const int i = i0 + 2 * tr;
+        const bool two_i = i + 1 < rows, two_j = j + 1 < M;
+        // (the rows of B and of the first columns are consecutive; c0 > 0: later columns, alone)
+        const int4* B = reinterpret_cast<const int4*>(sm.T + (M + i + c0) * ldm);
+        const int4* A = reinterpret_cast<const int4*>(sm.T + j);
+        const int lc = ldm >> 1, db = two_i ? lc : 0;
+        FullSum a0, a1, b0, b1;
 #pragma unroll 1
-        for (int k = 0; k < M; k += 2) {
-            const int4 x = pa[k >> 1], y = pb[k >> 1];
-            const int4 u = pc[k * lc], v = pc[(k + 1) * lc];
+        for (int k = 0; 2 * k < M; ++k) {
+            const int4 x = B[k], y = B[k + db], u = A[0], v = A[lc];
+            A += 2 * lc;
             const int2 x0 = make_int2(x.x, x.y), x1 = make_int2(x.z, x.w);
             const int2 y0 = make_int2(y.x, y.y), y1 = make_int2(y.z, y.w);
             const int2 u0 = make_int2(u.x, u.y), u1 = make_int2(u.z, u.w);
             const int2 v0 = make_int2(v.x, v.y), v1 = make_int2(v.z, v.w);
             a0.mac(x0, u0); a1.mac(x0, u1); b0.mac(y0, u0); b1.mac(y0, u1);
             a0.mac(x1, v0); a1.mac(x1, v1); b0.mac(y1, v0); b1.mac(y1, v1);
-            if ((k & 14) == 14) { a0.fold(); a1.fold(); b0.fold(); b1.fold(); }
+            if ((k & 7) == 7) { a0.fold(); a1.fold(); b0.fold(); b1.fold(); }
         }
-        auto put = [&](int i, int jj, const LimbSum& t) {
-            long long* d = fixed((i < s ? sm.C + i * ldm : sm.X + (i - s) * sm.ldx) + jj);
-            const long long v = *d - t.total();
-            *d = v;
-            if (i < s) top |= v ^ (v >> 63);
+        auto put = [&](int r, long long t0, long long t1) {
+            long long* d = fixed((r < s ? sm.C + r * ldm : sm.X + (r - s) * sm.ldx) + j);
+            t0 = d[0] - t0;
+            t1 = two_j ? d[1] - t1 : 0;
+            d[0] = t0;
+            if (two_j) d[1] = t1;
+            if (r < s) top |= (t0 ^ (t0 >> 63)) | (t1 ^ (t1 >> 63));
         };
-        put(ia, j, a0);
-        if (j + 1 < M) put(ia, j + 1, a1);
-        if (ib != ia) {
-            put(ib, j, b0);
-            if (j + 1 < M) put(ib, j + 1, b1);
-        }
+        put(i, a0.total(), a1.total());
+        if (two_i) put(i + 1, b0.total(), b1.total());
     }
     if (i0 < s) {  // the scale of C (one for all its rows)
         const int e = __reduce_max_sync(0xffffffffu, int_exp(top)) + eA + s_ns_eb + kSumUnit - 1;
@@ -612,7 +640,7 @@ __device__ __forceinline__ void ns_columns_to_limbs(int n, int M, int c0, int qk
     for (int c = threadIdx.x >> 5; c < qk; c += NT / 32) {
         double* X = sm.X + c * sm.ldx;
         const int eg = sm.eg[c0 + c];
-        const int u1 = eA + eg + kSumUnit - 1, u2 = eF - kFixBits;
+        const int u1 = eA + eg + kSumUnit - 1, u2 = eF - kPowerBits;
         int e1 = 0;
 #pragma unroll 1
         for (int t = lane; t < M; t += 32) e1 = max(e1, int_exp(fixed(X)[t]));
@@ -648,32 +676,28 @@ __device__ void ns_product_s(int n, int M, bool triangle, int c0, int qk, const 
     const int all = tri_tiles + ((qk + 1) >> 1) * nt;
 #pragma unroll 1
     for (int e = threadIdx.x; e < all; e += NT) {
-        int ia, ib, ja;
-        bool column = false;
-        if (e < tri_tiles) {
+        const bool column = e >= tri_tiles;
+        int I, J;
+        if (!column) {
             const int p = small_div(e, nt + 1), o = e - p * (nt + 1);
             const bool first = o <= p;
-            const int I = first ? p : nt - 1 - p, J = first ? o : o - p - 1;
+            I = first ? p : nt - 1 - p;
+            J = first ? o : o - p - 1;
             if (!first && I == p) continue;  // an odd middle row of tiles pairs with itself
-            ia = 2 * I;
-            ib = min(ia + 1, s - 1);
-            ja = 2 * J;
         } else {
-            const int t = e - tri_tiles, I = small_div(t, nt);
-            column = true;
-            ia = 2 * I;
-            ib = min(ia + 1, qk - 1);
-            ja = 2 * (t - I * nt);
+            I = small_div(e - tri_tiles, nt);
+            J = e - tri_tiles - I * nt;
         }
-        const int jb = min(ja + 1, s - 1);
-        auto b_of = [&](int i) { return reinterpret_cast<const int4*>(sm.T + (M + i) * ldm); };
-        auto c_of = [&](int i) { return reinterpret_cast<const int4*>(sm.C + i * ldm); };
-        const int4* Bia = column ? reinterpret_cast<const int4*>(sm.T + (n + c0 + ia) * ldm) : b_of(ia);
-        const int4* Bib = column ? reinterpret_cast<const int4*>(sm.T + (n + c0 + ib) * ldm) : b_of(ib);
-        const int4* Cia = column ? reinterpret_cast<const int4*>(sm.X + ia * sm.ldx) : c_of(ia);
-        const int4* Cib = column ? reinterpret_cast<const int4*>(sm.X + ib * sm.ldx) : c_of(ib);
-        const int4 *Bja = b_of(ja), *Bjb = b_of(jb), *Cja = c_of(ja), *Cjb = c_of(jb);
-        LimbSum aa, ab, ba, bb;
+        const int i = 2 * I, j = 2 * J;
+        const bool two_i = i + 1 < (column ? qk : s), two_j = j + 1 < s;
+        // the rows' first 16-byte words and the steps to their second rows
+        const int4* Bi = reinterpret_cast<const int4*>(sm.T + ((column ? n + c0 : M) + i) * ldm);
+        const int4* Ci = reinterpret_cast<const int4*>(column ? sm.X + i * sm.ldx : sm.C + i * ldm);
+        const int4* Bj = reinterpret_cast<const int4*>(sm.T + (M + j) * ldm);
+        const int4* Cj = reinterpret_cast<const int4*>(sm.C + j * ldm);
+        const int db = two_i ? ldm >> 1 : 0, dc = two_i ? (column ? sm.ldx : ldm) >> 1 : 0;
+        const int dj = two_j ? ldm >> 1 : 0;
+        FullSum aa, ab, ba, bb;
 #pragma unroll 1
         for (int k = 0; 2 * k < M; ++k) {
             auto half_step = [&](int4 bi, int4 bk, int4 cj, int4 ck) {
@@ -684,23 +708,19 @@ __device__ void ns_product_s(int n, int M, bool triangle, int c0, int qk, const 
                 aa.mac(x0, u0); ab.mac(x0, v0); ba.mac(y0, u0); bb.mac(y0, v0);
                 aa.mac(x1, u1); ab.mac(x1, v1); ba.mac(y1, u1); bb.mac(y1, v1);
             };
-            half_step(Bia[k], Bib[k], Cja[k], Cjb[k]);
-            half_step(Cia[k], Cib[k], Bja[k], Bjb[k]);
+            half_step(Bi[k], Bi[k + db], Cj[k], Cj[k + dj]);
+            half_step(Ci[k], Ci[k + dc], Bj[k], Bj[k + dj]);
             if ((k & 3) == 3) { aa.fold(); ab.fold(); ba.fold(); bb.fold(); }
         }
-        auto put = [&](int i, int j, const LimbSum& t) {
-            if (column) {
-                long long* d = fixed(sm.X) + i * sm.ldx + sm.x2 + j;
-                *d = *d - t.total();
-            } else if (j <= i) {
-                fixed(sm.S)[col_start(j, s) + i] = t.total();
-            }
-        };
-        put(ia, ja, aa);
-        if (jb != ja) put(ia, jb, ab);
-        if (ib != ia) {
-            put(ib, ja, ba);
-            if (jb != ja) put(ib, jb, bb);
+        // entry (i, j) and the steps to (i + 1, j) and (i, j + 1)
+        long long* d = column ? fixed(sm.X) + i * sm.ldx + sm.x2 + j : fixed(sm.S) + col_start(j, s) + i;
+        const int di = column ? sm.ldx : 1, dd = column ? 1 : s - j - 1;
+        const long long keep = column ? -1 : 0;  // S starts here
+        d[0] = (d[0] & keep) - aa.total();
+        if (two_j && (column || j < i)) d[dd] = (d[dd] & keep) - ab.total();
+        if (two_i) {
+            d[di] = (d[di] & keep) - ba.total();
+            if (two_j) d[di + dd] = (d[di + dd] & keep) - bb.total();
         }
     }
 }

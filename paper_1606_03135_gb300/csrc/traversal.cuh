@@ -1277,8 +1277,13 @@ __device__ void ns_coordinates(const SolveArgs& a, const Shape& sh, int j, const
 
 // Unit of the g rows in the elimination: 2^gs times the nodes' rows', so that ghat may reach
 // 8 2^gs: 64 at degree 2, 512, 1024 and 2048 at 3, 4 and 5, two to three times the largest
-// entries met in quasi-uniform, boundary and clustered stencils (24, 184, 439, 1023).
-__device__ __forceinline__ int ns_g_shift(int ell) { return ell < 2 ? 1 : (ell == 2 ? 3 : ell + 3); }
+// entries met in quasi-uniform, boundary and clustered stencils (24, 184, 439, 1023).  For a normal
+// derivative (kind 2, |g| <= 1) 8 to 128 is as wide; in the units of the Laplacians' its weights were
+// four times further from a double-double solve.
+__device__ __forceinline__ int ns_g_shift(int ell, int kind) {
+    if (kind == 2) return ell < 2 ? 0 : ell - 1;
+    return ell < 2 ? 1 : (ell == 2 ? 3 : ell + 3);
+}
 
 // The tableau of the constraints in fixed point (rows: nodes, then the q columns' right-hand sides
 // g).  kind 2: the normal derivative at the center of node j's own stencil (one column), else
@@ -1379,14 +1384,13 @@ __device__ __noinline__ bool ns_eliminate_fp64(const SolveArgs& a, const Shape& 
     return true;
 }
 
-// r^(m-2) and r^m of two stencil nodes as fractions of 2^(m-2) (kFixBits bits) and 2^m (kPowerBits:
-// the powers of near nodes, whose differences make the small eigenvalues of S, would lose with
-// fewer against the relative precision of FP64).  The squared
+// r^(m-2) and r^m of two stencil nodes as fractions of 2^(m-2) and 2^m with kPowerBits bits (the
+// powers of near nodes, whose differences make the small eigenvalues of S, would lose with fewer
+// against the relative precision of FP64).  The squared
 // distance is formed in FP64 without FMA, rounded as the oracle's (8 instructions in 3D; formed in
 // fixed point it took 48 others and made the weights two to five times closer to an exact solve, but
 // further from any FP64 one); its root and the powers of u = r / 2 <= 1 (the stencil's radius is 1)
 // in fixed point.
-constexpr int kPowerBits = 62;
 template <int D>
 __device__ __noinline__ void ns_powers(const double* xa, const double* xb, int m, long long* pm2,
                                        long long* pm) {
@@ -1397,14 +1401,13 @@ __device__ __noinline__ void ns_powers(const double* xa, const double* xb, int m
     unsigned long long u = ((unsigned long long)sqrt_core(N) << 2) >> min(1 - ((e - odd) >> 1), 63);
 #pragma unroll 1
     for (int s = 0; s < (m - 3) / 2; ++s) u = __umul64hi(u << 1, z);
-    *pm2 = shift_right((long long)u, kPowerBits - kFixBits);
+    *pm2 = (long long)u;
     *pm = (long long)__umul64hi(u << 1, z);
 }
 
-// coef r^(m-2) as a fraction of 2^(m-2+fs), coef <= 2^fs.
+// coef r^(m-2) as a fraction of 2^(m-2+fs) with kPowerBits bits, coef <= 2^fs.
 __device__ __forceinline__ long long ns_rhs_fixed(long long pm2, int coef, int fs) {
-    const int2 p = split_limbs(pm2);
-    return ((long long)p.x * coef << (kLimbBits - fs)) + (((long long)p.y * coef) >> fs);
+    return (((pm2 >> 32) * coef) << (32 - fs)) + (((pm2 & 0xffffffffll) * coef) >> fs);
 }
 
 // Scale of the columns' f rows: Laplacians reach coef 2^(m-2) (coef = m (m + D - 2) <= 2^fs), normal
@@ -1417,7 +1420,7 @@ __device__ __forceinline__ int ns_bits(int v) { return 32 - __clz(v - 1); }  // 
 // with them: the pairs of tableau rows with at least one basic node, (i, j) with j < M and i > j,
 // flattened by columns; f's entries at the other nodes of a column whose node is not basic either
 // start from zero (ns_finish adds them with A22).  A21 and f1 count 2^(m + scale of the row - 61) (the
-// unit of ns_product_c), f2 2^(m - 2 + fs - 58).  In integers throughout: about 200 issue slots
+// unit of ns_product_c), f2 2^(m - 2 + fs - 62).  In integers throughout: about 200 issue slots
 // per warp and pair, where the FP64 form has 14 FP64 instructions of 64 cycles each.
 template <int D, int NT>
 __device__ void ns_pairs(const Shape& sh, int q, int icoef, int fs, const NullSmem& sm) {
@@ -1454,7 +1457,7 @@ __device__ void ns_pairs(const Shape& sh, int q, int icoef, int fs, const NullSm
             for (int k = 0; k < 2; ++k) {  // f of column c at row r
                 const int c = k ? cb : ca, r = k ? i : j;
                 if (c < 0 || c >= q) continue;
-                fixed(sm.X)[c * sm.ldx + (r < M ? r : sm.x2 + r - M)] = r < M ? shift_fixed(f, fs + 1 - sm.eg[c]) : f;
+                fixed(sm.X)[c * sm.ldx + (r < M ? r : sm.x2 + r - M)] = r < M ? shift_fixed(f, fs - 3 - sm.eg[c]) : f;
             }
         }
     }
@@ -1495,12 +1498,12 @@ __device__ void ns_finish(const Shape& sh, int qk, int icoef, int fs, int kind, 
             const int ca = sm.colof[ra], cb = sm.colof[rb];
             if (kind != 2 && ((ca >= 0 && ca < qk) || (cb >= 0 && cb < qk))) {
                 const long long f = ns_rhs_fixed(pm2, icoef, fs);
-                const int u = eA - 2 + fs - kFixBits - kSumUnit - eC;  // of f, against 2^eg units
+                const int u = eA - 2 + fs - kPowerBits - kSumUnit - eC;  // of f, against 2^eg units
                 if (ca >= 0 && ca < qk) fixed(sm.X)[ca * sm.ldx + sm.x2 + j] += shift_fixed(f, u - sm.eg[ca]);
                 if (cb >= 0 && cb < qk) fixed(sm.X)[cb * sm.ldx + sm.x2 + i] += shift_fixed(f, u - sm.eg[cb]);
             }
         }
-        *d = from_fixed(a22 - *fixed(d), unit);
+        *d = from_fixed(a22 + *fixed(d), unit);
     }
 }
 
@@ -1520,15 +1523,14 @@ __device__ __forceinline__ void ns_rhs_to_fp64(int s, int c0, int qk, const Null
 // rho = f - A w in FP64 with the entries of A and f formed as the saddle-point systems form them
 // (correctly rounded coordinates, no FMA in the squared distances), then S dv = rho_other -
 // B rho_basic with the stored factors and w_basic -= B^T dv.  (The constraints hold by construction
-// and are left alone.)  It brings the weights to the error of an FP64 system.  That is an
-// improvement where r^m of most pairs is far below its scale, so that 58 bits of it are fewer than
-// FP64's: 3D stencils of degree 5 (M = 56; median error against a double-double solve 1.0e-11 ->
-// 5.9e-12, the refined saddle-point solve 6.2e-12); below that the unrefined weights are the better
-// ones (degree 4: 1.0e-12, refined 2.0e-12, saddle-point 1.9e-12).  So in plans that refine
-// (K >= 100) systems are refined whose pivots span at least 2^7 with M > 40, or 2^10 (3% of the
-// degree-4 stencils of a quasi-uniform ball, half of a strongly clustered cube's, where both are
-// equal), or every system with a.refine_all.  gw: scratch of 2 n words per column and n D words.
-__device__ __forceinline__ int ns_refine_log2(int M) { return M > 40 ? 7 : 10; }
+// and are left alone.)  Below a pivot span of 2^10 the unrefined weights are as close to a
+// double-double solve as refined ones (means over 60 stencils, unrefined / refined / refined
+// saddle-point solve: 3D ball, degree 5, 4.1e-12 / 3.9e-12 / 4.0e-12), from there on refinement
+// halves their error (clustered cube, degree 5, spans of 2^10 to 2^12: 9.5e-11 / 4.1e-11 /
+// 4.2e-11).  So in plans that refine (K >= 100) systems whose pivots span at least 2^10 are refined
+// (7% of the ball's, three quarters of the cube's), or every system with a.refine_all.  gw: scratch
+// of 2 n words per column and n D words.
+constexpr int kNullRefineLog2 = 10;
 
 template <int D, int NT>
 __device__ __noinline__ void ns_refine(const SolveArgs& a, const Shape& sh, int j, int c0, int qk,
@@ -1637,7 +1639,7 @@ __device__ __noinline__ void ns_refine(const SolveArgs& a, const Shape& sh, int 
 }
 
 // The columns c0 .. c0+qk-1 from their f rows on (the triangle's products and factorization with
-// the first chunk).  f counts 2^(eF - kFixBits).
+// the first chunk).  f counts 2^(eF - kPowerBits).
 template <int D, int NT, bool ALL_TEAMS>
 __device__ bool ns_columns(const SolveArgs& a, const Shape& sh, int j, int c0, int qk, int eF,
                            const NullSmem& sm, int kind) {
@@ -1668,7 +1670,7 @@ __device__ bool ns_columns(const SolveArgs& a, const Shape& sh, int j, int c0, i
     ns_basic_weights<NT>(n, M, c0, qk, sm);
     __syncthreads();
     if (double* gw = refine_scratch<NT, ALL_TEAMS>(a)) {
-        if (a.refine_all != 0 || s_ns_ratio >= ns_refine_log2(M))
+        if (a.refine_all != 0 || s_ns_ratio >= kNullRefineLog2)
             ns_refine<D, NT>(a, sh, j, c0, qk, sm, kind, gw);
     }
     return true;
@@ -1680,7 +1682,7 @@ __device__ bool ns_solve(const SolveArgs& a, const Shape& sh, int j, int q, int 
                          const NullSmem& sm, int kind) {
     const int tid = threadIdx.x, n = sh.n, M = sh.M;
     const int icoef = ns_coef<D>(sh), fs = ns_bits(icoef);
-    const int gs = ns_g_shift(sh.ell);
+    const int gs = ns_g_shift(sh.ell, kind);
     const int eg_min = fs - 3;  // f1 fits the unit of its products (ns_product_c)
     if (tid == 0) {
         s_ns_eb = 0;
@@ -1701,7 +1703,7 @@ __device__ bool ns_solve(const SolveArgs& a, const Shape& sh, int j, int q, int 
         for (int u = tid; u < n; u += NT) {
             const int p = sm.pos[u];
             fixed(sm.X)[p < M ? p : sm.x2 + p - M] =
-                to_fixed(neumann_at<D>(a, sh, j, u, sm.xi + u * D), p < M ? sh.m + sm.eg[0] + kSumUnit - 1 : sh.m - 2 + fs - kFixBits);
+                to_fixed(neumann_at<D>(a, sh, j, u, sm.xi + u * D), p < M ? sh.m + sm.eg[0] + kSumUnit - 1 : sh.m - 2 + fs - kPowerBits);
         }
         __syncthreads();
     }
@@ -1736,7 +1738,7 @@ __device__ __forceinline__ void ns_solve_chunk(const SolveArgs& a, const Shape& 
         long long pm2 = 0, pm;
         if (u != t) ns_powers<D>(sm.xi + u * D, sm.xi + t * D, sh.m, &pm2, &pm);
         const long long f = ns_rhs_fixed(pm2, icoef, fs);
-        fixed(sm.X)[c * sm.ldx + (p < M ? p : sm.x2 + p - M)] = p < M ? shift_fixed(f, fs + 1 - sm.eg[c0 + c]) : f;
+        fixed(sm.X)[c * sm.ldx + (p < M ? p : sm.x2 + p - M)] = p < M ? shift_fixed(f, fs - 3 - sm.eg[c0 + c]) : f;
     }
     __syncthreads();
     ns_columns<D, NT, false>(a, sh, j, c0, qk, sh.m - 2 + fs, sm, 0);

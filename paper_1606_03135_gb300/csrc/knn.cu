@@ -13,74 +13,70 @@
 namespace rbffd {
 
 // ------------------------------------------------------------------ exclusive scans
-// Single-CTA exclusive scan, out[0..count] with out[count] = total.  The input is walked in
-// tiles of 1024 x kScanCh elements: each tile is loaded and stored coalesced through shared
-// memory, where thread t scans its kScanCh contiguous elements; the block-wide scan of the
-// thread sums and the running total of earlier tiles give the offsets.  When count_dev is
-// given the element count is min(count, *count_dev), read on the device (the number of grid
-// cells in use is only known there).  Used for cell offsets and weight-slot offsets.
+// Single-CTA exclusive scan, out[0..count] with out[count] = total.  Each thread scans kScanCh
+// consecutive elements in registers (one 16-byte load), a warp its 128, and one barrier per tile of
+// 4096 hands round the warps' totals (two buffers in turn), which every warp sums for itself; the
+// next tile's elements are loaded before the barrier.  Bound by that chain of latencies (100,000
+// slot offsets from a cold cache: 56 us with tiles staged through shared memory and four barriers,
+// now 36).  Both arrays start on 16-byte boundaries.  When count_dev is given the element count is
+// min(count, *count_dev), read on the device (the number of grid cells in use is only known
+// there).  Used for cell offsets and weight-slot offsets.
 constexpr int kScanCh = 4;
 constexpr int kScanTile = 1024 * kScanCh;
-__device__ __forceinline__ int scan_pad(int e) { return e + (e >> 5); }  // fewer bank conflicts
 
-template <typename TI, typename TO>
-__global__ void __launch_bounds__(1024) k_scan(const TI* __restrict__ in, TO* __restrict__ out,
+__device__ __forceinline__ int4 scan_load(const int* __restrict__ in, int g, int count) {
+    if (g + kScanCh <= count) return *reinterpret_cast<const int4*>(in + g);
+    return make_int4(g < count ? in[g] : 0, g + 1 < count ? in[g + 1] : 0,
+                     g + 2 < count ? in[g + 2] : 0, 0);
+}
+
+template <typename TO>
+__global__ void __launch_bounds__(1024) k_scan(const int* __restrict__ in, TO* __restrict__ out,
                                                int count, const int* __restrict__ count_dev) {
-    __shared__ TO tile[kScanTile + kScanTile / 32];
-    __shared__ TO warp_tot[32];
+    __shared__ TO warp_tot[2][32];
     if (count_dev) count = min(count, *count_dev);
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     TO carry = 0;  // total of the earlier tiles (the same in every thread)
-    for (int base = 0; base < count; base += kScanTile) {
-#pragma unroll
-        for (int k = 0; k < kScanCh; ++k) {
-            const int e = k * 1024 + tid, g = base + e;
-            tile[scan_pad(e)] = g < count ? (TO)in[g] : (TO)0;
-        }
-        __syncthreads();
-        TO v[kScanCh], sum = 0;
-#pragma unroll
-        for (int k = 0; k < kScanCh; ++k) {
-            v[k] = tile[scan_pad(tid * kScanCh + k)];
-            sum += v[k];
-        }
+    int g = threadIdx.x * kScanCh, buf = 0;
+    int4 v = scan_load(in, g, count);
+    for (int base = 0; base < count; base += kScanTile, g += kScanTile, buf ^= 1) {
+        const TO v0 = v.x, v1 = v0 + v.y, v2 = v1 + v.z, sum = v2 + v.w;
         TO incl = sum;  // inclusive warp scan of the thread sums
         for (int o = 1; o < 32; o <<= 1) {
             const TO t = __shfl_up_sync(0xffffffffu, incl, o);
             if (lane >= o) incl += t;
         }
-        if (lane == 31) warp_tot[wid] = incl;
-        __syncthreads();
-        if (wid == 0) {
-            TO w = warp_tot[lane];
-            for (int o = 1; o < 32; o <<= 1) {
-                const TO t = __shfl_up_sync(0xffffffffu, w, o);
-                if (lane >= o) w += t;
+        if (lane == 31) warp_tot[buf][wid] = incl;
+        if (base + kScanTile < count) v = scan_load(in, g + kScanTile, count);
+        __syncthreads();  // (the other buffer was read before it)
+        TO w = warp_tot[buf][lane];  // inclusive over warps
+        for (int o = 1; o < 32; o <<= 1) {
+            const TO t = __shfl_up_sync(0xffffffffu, w, o);
+            if (lane >= o) w += t;
+        }
+        const TO before = __shfl_sync(0xffffffffu, w, max(wid - 1, 0));
+        const TO run = carry + (wid > 0 ? before : (TO)0) + (incl - sum);
+        carry += __shfl_sync(0xffffffffu, w, 31);
+        const TO r1 = run + v0, r2 = run + v1, r3 = run + v2;
+        if (g + kScanCh <= count) {
+            if constexpr (sizeof(TO) == 8) {
+                reinterpret_cast<longlong2*>(out + g)[0] = make_longlong2(run, r1);
+                reinterpret_cast<longlong2*>(out + g)[1] = make_longlong2(r2, r3);
+            } else {
+                *reinterpret_cast<int4*>(out + g) = make_int4(run, r1, r2, r3);
             }
-            warp_tot[lane] = w;  // inclusive over warps
+        } else {
+            if (g < count) out[g] = run;
+            if (g + 1 < count) out[g + 1] = r1;
+            if (g + 2 < count) out[g + 2] = r2;
         }
-        __syncthreads();
-        TO run = carry + (wid > 0 ? warp_tot[wid - 1] : (TO)0) + (incl - sum);
-#pragma unroll
-        for (int k = 0; k < kScanCh; ++k) {
-            tile[scan_pad(tid * kScanCh + k)] = run;
-            run += v[k];
-        }
-        carry += warp_tot[31];
-        __syncthreads();
-#pragma unroll
-        for (int k = 0; k < kScanCh; ++k) {
-            const int e = k * 1024 + tid, g = base + e;
-            if (g < count) out[g] = tile[scan_pad(e)];
-        }
-        __syncthreads();  // the next tile reuses tile[] and warp_tot[]
     }
-    if (tid == 0) out[count] = carry;
+    if (threadIdx.x == 0) out[count] = carry;
 }
 
 int launch_scan_i32_to_i64(const int* in, long long* out, int count, cudaStream_t s,
                            int* launches) {
-    k_scan<int, long long><<<1, 1024, 0, s>>>(in, out, count, nullptr);
+    k_scan<long long><<<1, 1024, 0, s>>>(in, out, count, nullptr);
     ++*launches;
     return RB_LAUNCHED(__func__);
 }
@@ -718,42 +714,47 @@ __global__ void __launch_bounds__(256) k_knn(const double* __restrict__ X, int N
 // Retention balls and traversal in-degrees of another delta from a plan's stencils (§4.1):
 // node q's closed ball of radius (1 - delta) rho_q is the prefix of its neighbour list with
 // d^2 <= (1 - delta)^2 rho_q^2, d^2 formed exactly as k_knn forms it (sqdist_rn of the same
-// coordinates, query first), so the balls equal the ones a new kNN pass would give.  One
-// warp per node; indeg must be zero on entry.
+// coordinates, query first), so the balls equal the ones a new kNN pass would give.  The list is
+// in the order of d^2: a thread per node finds the end of its prefix by bisection, seven FP64
+// distances per 32 nodes' lanes where a warp per node formed all n of them (16 cycles of the FP64
+// units an instruction; N = 100,000, n = 45: 121 us, now 31).  indeg must be zero on entry.
 template <int D>
-__global__ void __launch_bounds__(256) k_balls(const double* __restrict__ X, int N, int n,
+__global__ void __launch_bounds__(128) k_balls(const double* __restrict__ X, int N, int n,
                                                double omd2, const int* __restrict__ nbr,
                                                const double* __restrict__ rho2,
                                                const int* __restrict__ node_n,
                                                int* __restrict__ ball_len, int* __restrict__ indeg,
                                                DevCounters* ctr) {
     const int lane = threadIdx.x & 31;
-    const long long q = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (q >= N) return;  // (whole warps)
-    double xq[3];
-    for (int a = 0; a < D; ++a) xq[a] = X[q * D + a];
-    const int nq = node_n ? node_n[q] : n;
-    const double rball = __dmul_rn(omd2, rho2[q]);
-    const int* nb = nbr + q * n;
+    const int q = blockIdx.x * blockDim.x + threadIdx.x;
     int blen = 0;
-    for (int t0 = 0; t0 < nq; t0 += 32) {
-        const int t = t0 + lane;
-        bool inb = false;
-        if (t < nq) {
+    if (q < N) {
+        double xq[3];
+        for (int a = 0; a < D; ++a) xq[a] = X[(size_t)q * D + a];
+        const double rball = __dmul_rn(omd2, rho2[q]);
+        const int* nb = nbr + (size_t)q * n;
+        int end = node_n ? node_n[q] : n;  // the first neighbour outside lies in [blen, end]
+        while (blen < end) {
+            const int t = (blen + end) >> 1;
             const int id = nb[t];
             double xp[3];
             for (int a = 0; a < D; ++a) xp[a] = X[(size_t)id * D + a];
-            inb = sqdist_rn<D>(xq, xp) <= rball;
+            if (sqdist_rn<D>(xq, xp) <= rball) blen = t + 1;
+            else end = t;
         }
-        blen += __popc(__ballot_sync(0xffffffffu, inb));
-    }
-    if (lane == 0) {
         ball_len[q] = blen;
-        atomicMax(&ctr->max_ball, blen);
     }
-    for (int t = 1 + lane; t < blen; t += 32) {
-        const int i = nb[t];
-        if (i > q) atomicAdd(&indeg[i], 1);
+    const int longest = __reduce_max_sync(0xffffffffu, blen);
+    if (lane == 0) atomicMax(&ctr->max_ball, longest);
+    const int q0 = q - lane;
+#pragma unroll 4
+    for (int l = 0; l < 32; ++l) {
+        const int len = __shfl_sync(0xffffffffu, blen, l);  // (0 past the last node)
+        const int* nb = nbr + (size_t)(q0 + l) * n;
+        for (int t = 1 + lane; t < len; t += 32) {
+            const int i = nb[t];
+            if (i > q0 + l) atomicAdd(&indeg[i], 1);
+        }
     }
 }
 
@@ -802,7 +803,7 @@ static int grid_and_knn(const double* X, int N, int n, double omd2, void* scratc
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     k_grid_params<D><<<nb < sms ? nb : sms, tb, 0, s>>>(X, N, n, ncell_max, acc, gp);
     k_cell_count<D><<<nb, tb, 0, s>>>(X, N, gp, cell_of, count, rank);
-    k_scan<int, int><<<1, 1024, 0, s>>>(count, start, ncell_max, &gp->ncell);
+    k_scan<int><<<1, 1024, 0, s>>>(count, start, ncell_max, &gp->ncell);
     k_cell_fill<D><<<nb, tb, 0, s>>>(X, N, cell_of, start, rank, sorted_idx, sorted_X,
                                      sorted_Xf);
     const int wpb = 8;
@@ -836,8 +837,7 @@ int launch_balls(int D, const double* X, int N, int n, double omd2, const int* n
                  DevCounters* ctr, cudaStream_t s, int* launches) {
     int rc = RB_CUDA(cudaMemsetAsync(indeg, 0, (size_t)N * sizeof(int), s));
     if (rc) return rc;
-    const int tb = 256;
-    const unsigned nb = (unsigned)(((size_t)N * 32 + tb - 1) / tb);
+    const int tb = 128, nb = (N + tb - 1) / tb;
     if (D == 2) k_balls<2><<<nb, tb, 0, s>>>(X, N, n, omd2, nbr, rho2, node_n, ball_len, indeg, ctr);
     else k_balls<3><<<nb, tb, 0, s>>>(X, N, n, omd2, nbr, rho2, node_n, ball_len, indeg, ctr);
     ++*launches;

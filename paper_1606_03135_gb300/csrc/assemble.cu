@@ -401,13 +401,15 @@ static int pick_team(int lay, size_t smem, int force, int* nt_out, int* per_sm_o
     if (nt == 0 && lay == kNull) {
         // Null-space solves: a warp per system while at least 12 of them share an SM (enough warps
         // to hide each other's latency, no barriers), 128 threads down to five, 256 for two to
-        // four, 512 for one.  Traversal ms (32 / 64 / 96 / 128 threads): 3D ball N = 100k delta 1.0
-        // (14 systems per SM) 8.97 / 10.0 / 10.6 / 10.4, 0.4 (9) 6.58 / 6.13 / 5.97 / 5.78, 0.2 (6)
-        // 8.62 / 6.79 / 6.61 / 6.32; 2D square N = 40k delta 1.0 (22) 1.62 / 2.41 / 2.39 / 2.45, 0.3
-        // (12) 0.81 / 0.87 / 0.82 / 0.85; 2D degree 5 N = 30k delta 0.6 (12) 1.61 / 1.51 / - / 1.51.
+        // four, 512 for one.  Traversal ms (32 / 128 threads): 3D ball N = 100k delta 1.0 (16 systems
+        // per SM) 8.7 / 10.9, 0.4 (9) 6.7 / 6.1, 0.2 (6) 9.0 / 6.6; 2D square N = 40k delta 1.0 (22)
+        // 1.65 / 2.50, 0.3 (12) 0.82 / 0.87; 2D degree 5 N = 30k delta 0.6 (12) 1.65 / 1.54.  Plans that
+        // refine (not in 128-thread teams): 64 from six systems on, else 256: 3D degree 4 N = 12k
+        // delta 1.0 (6; 64 / 256) 3.9 / 4.4, 0.4 (3) 2.6 / 1.9.
         int per_sm = 0;
         if ((rc = occ(32, &per_sm))) return rc;
-        nt = per_sm >= 12 ? 32 : ((per_sm >= 5 && !refined) ? kNT : (per_sm >= 2 ? kMidNT : kMaxNT));
+        const bool many = refined ? per_sm >= 6 : per_sm >= 5;
+        nt = per_sm >= 12 ? 32 : (many ? (refined ? 64 : kNT) : (per_sm >= 2 ? kMidNT : kMaxNT));
     }
     if (nt == 0) {
         int per_sm = 0;

@@ -410,8 +410,9 @@ int plan_impl(const double* nodes, int64_t N, int d, int n, int ell, int m,
         Carver c;
         const size_t oX = c.add<double>((size_t)N * d), oN = c.add<int>((size_t)N * n),
                      oR = c.add<double>((size_t)N), oB = c.add<int>((size_t)N),
-                     oI = c.add<int>((size_t)N), oS = c.add<long long>((size_t)N + 1),
-                     oP = c.add<short>(basis_count), oC = c.add<DevCounters>(1),
+                     oI = c.add<int>((size_t)N), oP = c.add<short>(basis_count),
+                     oS = c.add<long long>((size_t)N + 1),  // (its total and the counters are
+                     oC = c.add<DevCounters>(1),            // read back together: side by side)
                      oNn = c.add<int>(mixed ? (size_t)N : 0),
                      oNl = c.add<signed char>(mixed ? (size_t)N : 0),
                      oNm = c.add<signed char>(mixed ? (size_t)N : 0),
@@ -480,13 +481,18 @@ int plan_impl(const double* nodes, int64_t N, int d, int n, int ell, int m,
     if (scratch) cudaFreeAsync(scratch, s);
     scratch = nullptr;
     {
-        long long slots = 0;  // pageable copies: each returns once the stream has reached it
-        if ((rc = bad(cudaMemcpyAsync(&p->h_ctr, p->ctr, sizeof(DevCounters),
-                                      cudaMemcpyDeviceToHost, s))) ||
-            (rc = bad(cudaMemcpyAsync(&slots, p->slot_off + N, sizeof(long long),
-                                      cudaMemcpyDeviceToHost, s))) ||
+        // One pageable copy (it returns once the stream has reached it, about 8 us) from the total
+        // of the slot offsets, their last entry, to the end of the counters.
+        const char* total = reinterpret_cast<const char*>(p->slot_off + N);
+        const size_t len = reinterpret_cast<const char*>(p->ctr + 1) - total;
+        char tail[sizeof(long long) + 256 + sizeof(DevCounters)];
+        long long slots = 0;
+        if (len > sizeof(tail)) { rc = RBFFD_EINVAL; goto fail; }  // (the carver pads below 256)
+        if ((rc = bad(cudaMemcpyAsync(tail, total, len, cudaMemcpyDeviceToHost, s))) ||
             (rc = bad(cudaStreamSynchronize(s))))
             goto fail;
+        memcpy(&slots, tail, sizeof(slots));
+        memcpy(&p->h_ctr, tail + len - sizeof(DevCounters), sizeof(DevCounters));
         p->total_slots = slots;
     }
     if (p->h_ctr.status) { rc = p->h_ctr.status; goto fail; }

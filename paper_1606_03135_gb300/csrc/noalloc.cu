@@ -69,8 +69,8 @@ extern "C" int rbffd_stencils_noalloc(const double* nodes, int64_t N, int d, int
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     int* indeg = reinterpret_cast<int*>(base + kGridBytes);
     DevCounters* ctr = reinterpret_cast<DevCounters*>(base + kGridBytes + kIndegBytes);
-    // the array keeps the previous call's contents: reset the status block (the grid counts,
-    // cursors and in-degrees are cleared inside the launch sequence)
+    // the array keeps the previous call's contents: reset the status block (the grid counts and
+    // in-degrees are cleared inside the launch sequence)
     if ((rc = RB_CUDA(cudaMemsetAsync(ctr, 0, sizeof(DevCounters), s)))) return rc;
     int launches = 0;
     rc = launch_grid_and_knn(d, nodes, Ni, n, (1.0 - delta) * (1.0 - delta), base, grid_bytes,

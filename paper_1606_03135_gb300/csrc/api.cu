@@ -528,11 +528,16 @@ int plan_impl(const double* nodes, int64_t N, int d, int n, int ell, int m,
         // r^7 and degree 5 the norms of their errors over a set's rows are 0.5 to 1.0 times its
         // (1.3 on a set whose largest error is one row's).  At degree 6 and above (the constraints'
         // pivots get small) and at r^9 and above (r^m spans more of the 58 bits) they are larger.
-        // Large systems (K >= 100, which refine) with n > 3 M are left out as well: S is nearly the
-        // whole matrix there (n = 128, M = 21: 5.0 ms against 5.35).  Those, plans of several
-        // shapes and systems too large for this layout factor the saddle-point matrix.
-        const bool null_space = ldlt && one_shape && 2 * ell + 1 >= m && m <= 7 && ell <= 5 &&
-                                (p->K < RBFFD_REFINE_MIN_K || n <= 3 * (p->K - n));
+        // Degree 5 with K < 100 (2D; not refined) keeps the saddle-point path although the null
+        // space is faster there (n = 43, N = 30k, delta 0.6: 1.6 against 2.55 ms): on sets with
+        // nearly coincident nodes that path's own error passes 1e-9 of the matrix's norm, so no
+        // other solver reproduces its matrix to that.  Large systems (K >= 100, which refine) with
+        // n > 3 M are left out as well: S is nearly the whole matrix there (n = 128, M = 21: 5.0 ms
+        // against 5.35).  Those, plans of several shapes and systems too large for this layout
+        // factor the saddle-point matrix.
+        const bool large = p->K >= RBFFD_REFINE_MIN_K;
+        const bool null_space = ldlt && one_shape && 2 * ell + 1 >= m && m <= 7 &&
+                                (large ? ell <= 5 && n <= 3 * (p->K - n) : ell <= 4);
         const int qcap0 = p->qcap;
         for (p->lay = null_space ? kLayNull : (ldlt ? kLayPacked : kLayFull);; p->lay = kLayPacked) {
             for (p->qcap = qcap0;; --p->qcap) {

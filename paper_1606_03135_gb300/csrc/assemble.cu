@@ -16,7 +16,7 @@
 // Local solve (one team of 32 to 512 threads per stencil).  The (n+M) x (n+M) saddle-point
 // matrix [A P; P^T 0] of §4.1 and the q right-hand sides of the overlapped system (one per
 // solved ball member) are formed in shared memory.  Plans whose stencils have one shape with
-// degree up to 5 and r^7 or below solve in the null space of P^T
+// degree up to 4 (5 for K >= 100) and r^7 or below solve in the null space of P^T
 // (nullspace.cuh: most of the work in fixed point on the integer pipe).  For the others the
 // lower triangle is stored packed and factored as L D L^T with Bunch-Kaufman pivoting, the
 // right-hand sides carried along ((1/3) K^3 + 2 K^2 q flops); the paper's
@@ -403,9 +403,9 @@ static int pick_team(int lay, size_t smem, int force, int* nt_out, int* per_sm_o
         // to hide each other's latency, no barriers), 128 threads down to five, 256 for two to
         // four, 512 for one.  Traversal ms (32 / 128 threads): 3D ball N = 100k delta 1.0 (16 systems
         // per SM) 8.7 / 10.9, 0.4 (9) 6.7 / 6.1, 0.2 (6) 9.0 / 6.6; 2D square N = 40k delta 1.0 (22)
-        // 1.65 / 2.50, 0.3 (12) 0.82 / 0.87; 2D degree 5 N = 30k delta 0.6 (12) 1.65 / 1.54.  Plans that
-        // refine (not in 128-thread teams): 64 from six systems on, else 256: 3D degree 4 N = 12k
-        // delta 1.0 (6; 64 / 256) 3.9 / 4.4, 0.4 (3) 2.6 / 1.9.
+        // 1.65 / 2.50, 0.3 (12) 0.82 / 0.87.  Plans that refine (not in 128-thread teams): 64 from
+        // six systems on, else 256: 3D degree 4 N = 12k delta 1.0 (6; 64 / 256) 3.9 / 4.4, 0.4 (3)
+        // 2.6 / 1.9.
         int per_sm = 0;
         if ((rc = occ(32, &per_sm))) return rc;
         const bool many = refined ? per_sm >= 6 : per_sm >= 5;

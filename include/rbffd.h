@@ -47,7 +47,10 @@ extern "C" {
 
 /* Factorization of the local symmetric saddle-point system (§4.1, §4.3 "one matrix
  * decomposition").  LDLT: symmetric indefinite LDL^T with Bunch-Kaufman pivoting,
- * (1/3) K^3 flops; LU: partial-pivot LU, (2/3) K^3 flops.  Same weights up to rounding. */
+ * (1/3) K^3 flops, or, for plans of one stencil shape with r^7 or below, 2 degree + 1 >= the
+ * exponent, and degree up to 4, or K >= 100, n <= 3 M and degree up to 5, an LDL^T of the system
+ * reduced to the null space of the polynomial constraints (as accurate, most of it in fixed point);
+ * LU: partial-pivot LU, (2/3) K^3 flops.  Same weights up to rounding. */
 #define RBFFD_FACTOR_LDLT 0
 #define RBFFD_FACTOR_LU 1
 
@@ -71,10 +74,11 @@ typedef struct {
     int max_ctas;       /* cap on the persistent traversal grid, so that plans assembled
                            concurrently on several streams share the GPU; 0 = fill the GPU */
     int team;           /* threads per stencil team: 0 = chosen from the shared-memory
-                           footprint (96 for LDL^T, or 128 if that keeps more stencils
-                           resident, when more than 4 fit an SM and the plan does not
-                           refine; 256 when 2 to 4 fit, or more for a plan that refines;
-                           512 when one fits), or 32 (one warp per stencil), 64, 96, 128,
+                           footprint (null-space systems: 32 when 12 or more fit an SM;
+                           otherwise, when more than 4 fit an SM and the plan does not
+                           refine, 128, or 96 for the saddle-point LDL^T unless that keeps
+                           fewer resident; 256 when 2 to 4 fit, or more for a plan that
+                           refines; 512 when one fits), or 32 (one warp per stencil), 64, 96, 128,
                            256 or 512 to force one (used by the schedule autotuner); 32, 64,
                            96 and 256 need RBFFD_FACTOR_LDLT, else RBFFD_EINVAL; 96 and 128
                            are refused for plans that refine (see refine) */
@@ -93,12 +97,13 @@ typedef struct {
                            stencils in 3D reach condition numbers near 1e10, where the first
                            solution's error is dominated by the symmetric-pivoting
                            factorization): RBFFD_REFINE_AUTO (default) refines a system when its
-                           pivots span at least 2^16 (max |d| / min |d| over the D blocks, a
-                           lower bound of its condition number); RBFFD_REFINE_ALL refines every
+                           pivots span at least 2^16, in the null space 2^10 (max |d| / min |d|
+                           over the D blocks, a lower bound of its condition number); RBFFD_REFINE_ALL refines every
                            system of every plan; RBFFD_REFINE_NONE none.  The residual b - A x0 is formed
                            in FP64 with the assembled system (copied to the plan's assembly
                            memory before the factorization: one full K x K copy per resident
-                           CTA) and the correction is solved with
+                           CTA; in the null space its entries are formed again) and the
+                           correction is solved with
                            the stored factors (about 4 K^2 flops per refined column).  With a
                            Lebesgue test (SEQ, FALLBACK) a column whose first Lebesgue value
                            exceeds the test's reference by more than 2^-10 of it is not

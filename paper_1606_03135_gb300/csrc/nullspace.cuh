@@ -334,12 +334,16 @@ static __device__ __noinline__ long long row_dot_col(const double* row, const do
 // the rank-1 form of Gauss-Jordan elimination, one rounding per term, took about 30.
 //
 // Units: 2^-kTabBits for P, U, L and B, times 2^gs for the rows of g (gs from the degree); entries
-// must stay below 2^59 units (8, and 8 2^gs).  Thin or nearly degenerate stencils that leave this
-// range are noticed and done again in FP64.  Returns 1, 0 on an exactly zero pivot column, -1 on a
-// range (uniformly).  On return the rows of B and ghat are limbs at the scales s_ns_eb (once the
-// team has met) and sm.eg (at least eg_min; a row's absolute sum stays below 4 times its scale,
-// which bounds the products' sums).
-constexpr int kTabBits = 56;
+// must stay below 2^59 units (8, and 8 2^gs), pivots at least 2^-kPivotBits: a column's entries are
+// held to 2^-57, so a small pivot has few bits left, and one below the unit would look like an exact
+// zero (flat stencils, whose monomials z^k are small: with pivots near 2^-18 the weights of degree 2
+// would be 30 times further off than the coordinates' rounding puts them, from 2^-12 on they are
+// not).  Quasi-uniform, boundary and clustered stencils of degree 2 to 5 have pivots of 2^-9 and
+// more.  Stencils that leave these ranges are noticed and done again in FP64, which alone decides
+// that a pivot is zero.  Returns false on a range (uniformly).  On return the rows of B and ghat
+// are limbs at the scales s_ns_eb (once the team has met) and sm.eg (at least eg_min; a row's
+// absolute sum stays below 4 times its scale, which bounds the products' sums).
+constexpr int kTabBits = 56, kPivotBits = 12;
 
 __device__ __forceinline__ bool limb_overflow(long long v) {
     const int hi = (int)(v >> 32);
@@ -347,9 +351,10 @@ __device__ __forceinline__ bool limb_overflow(long long v) {
 }
 
 template <int NT>
-__device__ int ns_eliminate_fixed(int n, int M, int q, int gs, int eg_min, const NullSmem& sm) {
+__device__ bool ns_eliminate_fixed(int n, int M, int q, int gs, int eg_min, const NullSmem& sm) {
     __shared__ long long s_y;
     __shared__ int s_sh, s_piv;
+    constexpr unsigned kLeast = 1u << (kTabBits - kPivotBits - 28);  // in the search's 2^28 units
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int ldm = sm.ldm, R = n + q;
     double* T = sm.T;
@@ -374,7 +379,7 @@ __device__ int ns_eliminate_fixed(int n, int M, int q, int gs, int eg_min, const
             }
             const unsigned top = __reduce_max_sync(0xffffffffu, best);
             p = (int)__reduce_min_sync(0xffffffffu, best == top ? (unsigned)p : 0x7fffffffu);
-            if (top == 0u) p = -1;
+            if (top < kLeast) p = -1;
             if (p > k) {
 #pragma unroll 1
                 for (int c = lane; c < M; c += 32) {
@@ -389,13 +394,13 @@ __device__ int ns_eliminate_fixed(int n, int M, int q, int gs, int eg_min, const
             const unsigned long long a = (unsigned long long)(d < 0 ? -d : d);
             const int lz = __clzll((long long)a);
             if constexpr (NT == 32) {
-                if (p < 0) return 0;
+                if (p < 0) return false;
             }
             const long long y = rcp_norm(a << (lz & 63));
             if (lane == 0) { s_y = d < 0 ? -y : y; s_sh = lz; s_piv = p; }
         }
         team_sync<NT>();
-        if (NT > 32 && s_piv < 0) return 0;
+        if (NT > 32 && s_piv < 0) return false;
         const int2 y = split_limbs(s_y);
         const int lz = s_sh;
         // 1 / d = y 2^(lz - 121): the multiplier v / d in 2^-56 is mul_limbs(v 2^e, y) 2^(lz - 9 - e)
@@ -462,7 +467,7 @@ __device__ int ns_eliminate_fixed(int n, int M, int q, int gs, int eg_min, const
                 for (int k = 0; k < M; ++k) limbs(row)[k] = split_limbs(shift_fixed(join_limbs(limbs(row)[k]), e0 - eg));
         }
     }
-    if (__syncthreads_or(bad)) return -1;
+    if (__syncthreads_or(bad)) return false;
     const int sh = kFixBits - kTabBits - s_ns_eb;
     if (sh < 0) {
 #pragma unroll 1
@@ -471,10 +476,10 @@ __device__ int ns_eliminate_fixed(int n, int M, int q, int gs, int eg_min, const
             for (int k = 0; k < M; ++k)
                 limbs(T)[i * ldm + k] = split_limbs(shift_fixed(join_limbs(limbs(T)[i * ldm + k]), sh));
     }
-    return 1;
+    return true;
 }
 
-// The same three steps in FP64.
+// The same three steps in FP64.  Returns false on an exactly zero pivot column.
 template <int NT>
 __device__ bool ns_eliminate(int n, int M, int q, const NullSmem& sm) {
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;

@@ -1691,8 +1691,9 @@ __device__ bool ns_solve(const SolveArgs& a, const Shape& sh, int j, int q, int 
     ns_coordinates<D, NT>(a, sh, j, sm);
     __syncthreads();
     ns_constraints_fixed<D, NT>(a, sh, j, q, gs, sm, kind);
-    const int done = ns_eliminate_fixed<NT>(n, M, q, gs, eg_min, sm);
-    if (done == 0 || (done < 0 && !ns_eliminate_fp64<D, NT>(a, sh, j, q, eg_min, sm, kind))) return false;
+    if (!ns_eliminate_fixed<NT>(n, M, q, gs, eg_min, sm) &&
+        !ns_eliminate_fp64<D, NT>(a, sh, j, q, eg_min, sm, kind))
+        return false;
 #pragma unroll 1
     for (int t = tid; t < n; t += NT) sm.pos[sm.order[t]] = t;
     __syncthreads();

@@ -1375,6 +1375,7 @@ __device__ void ns_constraints(const SolveArgs& a, const Shape& sh, int j, int q
 template <int D, int NT>
 __device__ __noinline__ bool ns_eliminate_fp64(const SolveArgs& a, const Shape& sh, int j, int q,
                                                int eg_min, const NullSmem& sm, int kind) {
+    if (threadIdx.x == 0) s_ns_eb = 0;  // (rows that left the fixed-point range may have raised it)
     ns_constraints<D, NT>(a, sh, j, q, sm, kind);
     if (!ns_eliminate<NT>(sh.n, sh.M, q, sm)) return false;
     ns_scales<NT>(sh.n, sh.M, q, eg_min, sm);

@@ -59,7 +59,11 @@ struct rbffd_plan_s {
     int refine_min_K = 0x7fffffff;  // systems with K >= this are refined
     long long rs_doubles = 0, rs_stride = 0;  // refinement scratch: size, per traversal CTA
     int rs_x0 = 0;                  // offset of the first solution within a slot
+    long long sd_stride = 0;        // null-space plans: bytes of a saddle-point block
+    int sd_slots = 0;               // and how many there are
     double* rs = nullptr;
+    char* sd = nullptr;
+    int* sd_lock = nullptr;
     // traversal and results
     bool have_asm = false, assembled = false;
     int* state = nullptr;
@@ -594,6 +598,21 @@ int plan_impl(const double* nodes, int64_t N, int d, int n, int ell, int m,
             p->rs_doubles = doubles;
             p->asm_bytes += ((size_t)doubles * 8 + 255) & ~size_t(255);
         }
+        if (p->lay == kLayNull) {
+            // saddle-point blocks: one per CTA up to 512 of them and 8 MB (24 MB in plans that
+            // refine, whose systems are larger), shared by the CTAs beyond that
+            p->sd_stride = (long long)((solve_smem_per_cta(n, p->K, kSaddleCols, kSaddleCols, d, kLayPacked,
+                                                           nullptr) + 255) & ~size_t(255));
+            const long long fit = (p->K >= p->refine_min_K ? 24ll << 20 : 8ll << 20) / p->sd_stride;
+            long long most = p->lp.grid > p->lp.fb[0].grid ? p->lp.grid : p->lp.fb[0].grid;
+            if (most > 512) most = 512;
+            if (most > N) most = N;
+            p->sd_slots = (int)(most < fit ? most : fit);
+            Carver c;
+            c.add<char>((size_t)p->sd_slots * p->sd_stride);
+            c.add<int>(p->sd_slots);
+            p->asm_bytes += c.bytes;
+        }
     }
     *out = p;
     return RBFFD_OK;
@@ -669,7 +688,9 @@ int rbffd_assemble(rbffd_plan_t p, void* stream, rbffd_csr* out) {
                      o_rp = c.add<long long>(N + 1), o_col = c.add<int>(N * n),
                      o_val = c.add<double>(N * n), o_lam = c.add<double>(N),
                      o_isc = c.add<unsigned char>(N), o_spec = c.add<int>(N),
-                     o_rs = c.add<double>((size_t)p->rs_doubles);
+                     o_rs = c.add<double>((size_t)p->rs_doubles),
+                     o_sd = c.add<char>((size_t)p->sd_slots * p->sd_stride),
+                     o_sdl = c.add<int>(p->sd_slots);
         if ((rc = pool_alloc(&p->asm_block, c.bytes, p->device, s))) return rc;
         void* b = p->asm_block;
         p->state = at<int>(b, o_state); p->pending = at<int>(b, o_pend);
@@ -681,6 +702,8 @@ int rbffd_assemble(rbffd_plan_t p, void* stream, rbffd_csr* out) {
         p->lam_row = at<double>(b, o_lam); p->is_center = at<unsigned char>(b, o_isc);
         p->spec = at<int>(b, o_spec);
         p->rs = p->rs_doubles > 0 ? at<double>(b, o_rs) : nullptr;
+        p->sd = at<char>(b, o_sd);
+        p->sd_lock = at<int>(b, o_sdl);
         p->have_asm = true;
     }
     SolveArgs a{};
@@ -709,6 +732,10 @@ int rbffd_assemble(rbffd_plan_t p, void* stream, rbffd_csr* out) {
     a.fma_r2 = p->rs == nullptr ? 1 : 0;  // (saddle-point layouts)
     a.rs_stride = p->rs_stride;
     a.rs_x0 = p->rs_x0;
+    a.sd = p->sd;
+    a.sd_stride = p->sd_stride;
+    a.sd_lock = p->sd_lock;
+    a.sd_slots = p->sd_slots;
     a.refine_min_K = p->refine_min_K;
     a.refine_all = p->opts.refine == RBFFD_REFINE_ALL ? 1 : 0;
 

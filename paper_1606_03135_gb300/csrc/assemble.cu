@@ -58,7 +58,8 @@ size_t basis_smem_bytes(int count) { return ((size_t)count * sizeof(short) + 15)
 
 __global__ void k_traversal_init(int N, const int* __restrict__ indeg,
                                  const unsigned char* __restrict__ bc, int* state, int* pending,
-                                 int* owner, int* queue, unsigned char* fb_flag, int* spec) {
+                                 int* owner, int* queue, unsigned char* fb_flag, int* spec,
+                                 int* sd_lock, int sd_slots) {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) {
         state[i] = (bc && bc[i]) ? kBoundary : kUndecided;
         if (spec) spec[i] = 0;
@@ -66,6 +67,7 @@ __global__ void k_traversal_init(int N, const int* __restrict__ indeg,
         owner[i] = kNoOwner;
         queue[i] = -1;
         fb_flag[i] = 0;
+        if (i < sd_slots) sd_lock[i] = 0;  // (sd_slots <= N)
     }
 }
 
@@ -472,7 +474,7 @@ static int traversal(const SolveArgs& a, const LaunchPlan& lp, const int* indeg,
     const int basis_bytes = (int)basis_smem_bytes(a.basis_count);
     const int tb = 256, nb = (a.N + tb - 1) / tb;
     k_traversal_init<<<nb, tb, 0, s>>>(a.N, indeg, a.bc, a.state, a.pending, a.owner, a.queue,
-                                       a.fb_flag, a.spec);
+                                       a.fb_flag, a.spec, a.sd_lock, a.sd_slots);
     if (a.bc) {
         k_boundary_release<<<nb, tb, 0, s>>>(a);
         ++*launches;

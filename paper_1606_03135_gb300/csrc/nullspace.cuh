@@ -339,8 +339,7 @@ static __device__ __noinline__ long long row_dot_col(const double* row, const do
 // zero (flat stencils, whose monomials z^k are small: with pivots near 2^-18 the weights of degree 2
 // would be 30 times further off than the coordinates' rounding puts them, from 2^-12 on they are
 // not).  Quasi-uniform, boundary and clustered stencils of degree 2 to 5 have pivots of 2^-9 and
-// more.  Stencils that leave these ranges are noticed and done again in FP64, which alone decides
-// that a pivot is zero.  Returns false on a range (uniformly).  On return the rows of B and ghat
+// more.  Stencils that leave these ranges are noticed and done again in FP64.  Returns false on a range (uniformly).  On return the rows of B and ghat
 // are limbs at the scales s_ns_eb (once the team has met) and sm.eg (at least eg_min; a row's
 // absolute sum stays below 4 times its scale, which bounds the products' sums).
 constexpr int kTabBits = 56, kPivotBits = 12;
@@ -479,12 +478,26 @@ __device__ bool ns_eliminate_fixed(int n, int M, int q, int gs, int eg_min, cons
     return true;
 }
 
-// The same three steps in FP64.  Returns false on an exactly zero pivot column.
+// The same three steps in FP64.  Returns false on a column that depends on the earlier ones: its
+// largest entry left is below 2^-kRankBits of its largest one before (in sm.X).  Lattices have such
+// columns, as polynomials that vanish at all of a stencil's nodes: rounding leaves up to 2^-49 of
+// them, and 2^-34 with nodes 2^15 radii from the origin.  Thin stencils along an axis keep 2^-8,
+// slabs of 1:1000 across the axes 2^-31.
+constexpr int kRankBits = 34;
+
 template <int NT>
 __device__ bool ns_eliminate(int n, int M, int q, const NullSmem& sm) {
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int ldm = sm.ldm, R = n + q;
     double* T = sm.T;
+#pragma unroll 1
+    for (int c = tid; c < M; c += NT) {
+        double top = 0.0;
+#pragma unroll 1
+        for (int i = 0; i < n; ++i) top = mag_key(T[i * ldm + c]) > mag_key(top) ? T[i * ldm + c] : top;
+        sm.X[c] = top;
+    }
+    __syncthreads();
 #pragma unroll 1
     for (int k = 0; k < M; ++k) {
         if (wid == 0) {
@@ -497,7 +510,9 @@ __device__ bool ns_eliminate(int n, int M, int q, const NullSmem& sm) {
             }
             const unsigned top = __reduce_max_sync(0xffffffffu, best);
             p = (int)__reduce_min_sync(0xffffffffu, best == top ? (unsigned)p : 0x7fffffffu);
-            if (top != 0u) {
+            // (exponents of the two magnitudes; a zero column has none left)
+            const bool left = top != 0u && (int)(mag_key(sm.X[k]) >> 20) - (int)(top >> 20) < kRankBits;
+            if (left) {
                 if (p != k) {
 #pragma unroll 1
                     for (int c = lane; c < M; c += 32) {
@@ -512,7 +527,7 @@ __device__ bool ns_eliminate(int n, int M, int q, const NullSmem& sm) {
 #pragma unroll 1
                 for (int i = k + 1 + lane; i < R; i += 32) T[i * ldm + k] *= rcp;
             }
-            if (lane == 0) s_ns_ok = top != 0u;
+            if (lane == 0) s_ns_ok = left;
         }
         __syncthreads();
         if (!s_ns_ok) return false;
@@ -736,10 +751,17 @@ __device__ void ns_product_s(int n, int M, bool triangle, int c0, int qk, const 
 // j = 0, 1, ... (L_pj = w_pj / d_j), in two forms with the same operations: a single warp goes
 // left-looking, a row (of S or of a column) per lane and one dot product per column, which takes
 // three instructions per FMA; larger teams, which hold large systems, go right-looking, all
-// threads sharing each update.  Returns false on an exactly zero pivot.
+// threads sharing each update.  Returns false on a pivot below 2^-kSpanBits of the largest one (S is
+// definite, so that is rounding: nodes too near each other).
 // s_ns_ratio: floor(log2) of the largest over that of the smallest pivot, a lower bound of S's
 // condition number (read after a barrier).
 __shared__ int s_ns_ratio;
+constexpr int kSpanBits = 49;
+
+// (d_max: the largest key so far, d among them)
+__device__ __forceinline__ bool pivot_lost(double d, unsigned d_max) {
+    return abs_bits(d) == 0ull || (int)(d_max >> 20) - (int)(mag_key(d) >> 20) > kSpanBits;
+}
 
 template <int NT>
 __device__ bool ns_factor(int s, int qk, const NullSmem& sm) {
@@ -772,9 +794,9 @@ __device__ bool ns_factor(int s, int qk, const NullSmem& sm) {
                 if (r == lane) d = v;
             }
             d = __shfl_sync(0xffffffffu, d, 0);
-            if (abs_bits(d) == 0ull) return false;
-            const double rcp = rcp_fixed(d);
             d_max = max(d_max, mag_key(d));
+            if (pivot_lost(d, d_max)) return false;
+            const double rcp = rcp_fixed(d);
             d_min = min(d_min, mag_key(d));
             if (lane == 0) sm.rd[p] = rcp;
             __syncwarp();
@@ -785,9 +807,9 @@ __device__ bool ns_factor(int s, int qk, const NullSmem& sm) {
             if (wid == 0) {
                 const double d = S[col_start(p, s) + p];
                 const double rcp = rcp_fixed(d);
-            d_max = max(d_max, mag_key(d));
-            d_min = min(d_min, mag_key(d));
-                if (lane == 0) { sm.rd[p] = rcp; s_ns_ok = abs_bits(d) != 0ull; }
+                d_max = max(d_max, mag_key(d));
+                d_min = min(d_min, mag_key(d));
+                if (lane == 0) { sm.rd[p] = rcp; s_ns_ok = !pivot_lost(d, d_max); }
 #pragma unroll 1
                 for (int i = p + 1 + lane; i < s; i += 32) sm.wb[i] = S[col_start(p, s) + i] * rcp;
             }

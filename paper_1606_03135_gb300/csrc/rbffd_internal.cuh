@@ -175,6 +175,14 @@ struct SolveArgs {
     int refine_all;            // 1: refine every system; 0: only those whose pivot ratio
                                // max |d| / min |d| reaches 2^16 (ill-conditioned)
 
+    // Null-space plans: sd_slots blocks of sd_stride bytes at sd, one saddle-point system with
+    // kSaddleCols right-hand sides each, for the stencils that the null space cannot solve, and a
+    // lock per block (0: free).
+    char* sd;
+    long long sd_stride;
+    int* sd_lock;
+    int sd_slots;
+
     unsigned long long timeout_ns;
     // traversal state
     int* state;
@@ -193,6 +201,7 @@ struct SolveArgs {
 // Layout of the local systems of a plan: the full matrix (LU), the packed lower triangle
 // (LDL^T), or the null space of the polynomial constraints (nullspace.cuh).
 constexpr int kLayFull = 0, kLayPacked = 1, kLayNull = 2;
+constexpr int kSaddleCols = 4;  // right-hand sides of a saddle-point block of a null-space plan
 
 size_t solve_smem_per_cta(int n, int K, int qcap, int qmax, int D, int lay, int* stride_out);
 // Kernels of nullspace.cu by team size (nullptr: no such team).

@@ -1004,6 +1004,13 @@ __device__ __forceinline__ double neumann_value(const SolveArgs& a, const Shape&
     return neumann_at<D>(a, sh, i, u, xi + (u < sh.n ? u * D : 0));
 }
 
+// Normal-derivative right-hand side of node i's own stencil, replacing column 0 of the
+// right-hand-side block (unknowns in index order, before the factorization).
+template <int D, int NT>
+__device__ void neumann_rhs(const SolveArgs& a, const Shape& sh, int i, const StencilSmem& sm) {
+    for (int j = threadIdx.x; j < sh.n + sh.M; j += NT) sm.X[j * sm.xs] = neumann_value<D>(a, sh, i, j, sm.xi);
+}
+
 // Team sizes whose traversal kernels carry the refinement step: the 96- and 128-thread teams
 // run with 40 registers for small systems (many per SM), and the planner gives plans that
 // refine (largest system K >= 100, at most a few per SM) 256- or 512-thread teams, or 32 or
@@ -1639,6 +1646,89 @@ __device__ __noinline__ void ns_refine(const SolveArgs& a, const Shape& sh, int 
     __syncthreads();
 }
 
+// Acquire-release fence at device scope: orders this thread's earlier memory operations, and
+// those of its CTA that a barrier made visible to it, before its later ones, as seen by every
+// thread of the device.  Only threads that publish (or consume) traversal state execute it.
+__device__ __forceinline__ void fence_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
+
+// The columns c0 .. c0+qk-1 of a stencil that the null space cannot solve, from its saddle-point
+// system like the plans of the other layouts (unrefined): constraints that depend on each other, as
+// on lattices, or a pivot of S at the level of its rounding (nodes within about 1e-8 of their
+// distance to the others).  The system lies in one of the plan's blocks in global memory, taken for
+// the time of the solve (whoever holds one waits for nobody); the columns go through it kSaddleCols
+// at a time, and their weights to the places that ns_weight reads.  False on an exactly zero pivot.
+__shared__ int s_ns_saddle;  // this stencil's columns come from here
+
+template <int D, int NT>
+__device__ __noinline__ bool saddle_columns(const SolveArgs& a, const Shape& sh, int j, int c0, int qk,
+                                            const NullSmem& sm, int kind) {
+    __shared__ int s_block;
+    const int tid = threadIdx.x, n = sh.n, M = sh.M, K = sh.K;
+    if (tid == 0) {
+        const unsigned long long t0 = globaltimer_ns();
+        int b = (int)(blockIdx.x % (unsigned)a.sd_slots);
+        while (atomicCAS(&a.sd_lock[b], 0, 1) != 0) {
+            b = b + 1 == a.sd_slots ? 0 : b + 1;
+            if (globaltimer_ns() - t0 > a.timeout_ns) {
+                set_error(a.ctr, RBFFD_ETIMEOUT);
+                b = -1;
+                break;
+            }
+            __nanosleep(64);
+        }
+        fence_gpu();  // (its last holder is done with it)
+        s_block = b;
+        s_ns_saddle = 1;
+    }
+    __syncthreads();
+    const int block = s_block;
+    if (block < 0) return false;
+    StencilSmem st;
+    carve<D, true>(a.sd + (size_t)block * a.sd_stride, a.n, a.K, kSaddleCols, kSaddleCols | 1, st);
+    bool ok = true;
+#pragma unroll 1
+    for (int b = 0; b < qk && ok; b += kSaddleCols) {
+        const int q = min(kSaddleCols, qk - b), first = c0 + b;
+#pragma unroll 1
+        for (int t = tid; t < n; t += NT) {
+            const int c = sm.colof[t] - first;
+            st.colof[t] = c >= 0 && c < q ? c : -1;
+        }
+        if (tid < q) st.cols[tid] = sm.cols[first + tid];
+        __syncthreads();
+        if (b == 0) {
+            assemble_local<D, true, NT>(a, sh, j, q, st);
+            if (kind == 2) {
+                neumann_rhs<D, NT>(a, sh, j, st);
+                __syncthreads();
+            }
+            ok = factor_solve_ldlt<NT>(K, q, st);
+        } else {
+            chunk_rhs<D, NT>(sh, 0, q, st, a.fma_r2 != 0);
+            __syncthreads();
+            forward_subst<NT>(K, q, st);
+            ldlt_solve_tail<NT>(K, q, st);
+        }
+        __syncthreads();
+#pragma unroll 1
+        for (int e = tid; ok && e < q * n; e += NT) {
+            const int c = small_div(e, n), r = e - c * n;
+            const double w = st.X[st.rowof[r] * st.xs + c];
+            if (r < M) sm.T[(n + first + c) * sm.ldm + r] = w;
+            else sm.X[(b + c) * sm.ldx + sm.x2 + r - M] = w;
+        }
+        __syncthreads();
+    }
+#pragma unroll 1
+    for (int t = tid; t < n; t += NT) sm.pos[t] = t;
+    if (tid == 0) {
+        fence_gpu();
+        atomicExch(&a.sd_lock[block], 0);
+    }
+    __syncthreads();
+    return ok;
+}
+
 // The columns c0 .. c0+qk-1 from their f rows on (the triangle's products and factorization with
 // the first chunk).  f counts 2^(eF - kPowerBits).
 template <int D, int NT, bool ALL_TEAMS>
@@ -1688,13 +1778,14 @@ __device__ bool ns_solve(const SolveArgs& a, const Shape& sh, int j, int q, int 
     if (tid == 0) {
         s_ns_eb = 0;
         s_ns_ec = sh.m - 2;  // A22 (scale 2^m) fits the unit of the sums
+        s_ns_saddle = 0;
     }
     ns_coordinates<D, NT>(a, sh, j, sm);
     __syncthreads();
     ns_constraints_fixed<D, NT>(a, sh, j, q, gs, sm, kind);
     if (!ns_eliminate_fixed<NT>(n, M, q, gs, eg_min, sm) &&
         !ns_eliminate_fp64<D, NT>(a, sh, j, q, eg_min, sm, kind))
-        return false;
+        return saddle_columns<D, NT>(a, sh, j, 0, q1, sm, kind);
 #pragma unroll 1
     for (int t = tid; t < n; t += NT) sm.pos[sm.order[t]] = t;
     __syncthreads();
@@ -1709,7 +1800,8 @@ __device__ bool ns_solve(const SolveArgs& a, const Shape& sh, int j, int q, int 
         }
         __syncthreads();
     }
-    return ns_columns<D, NT, ALL_TEAMS>(a, sh, j, 0, q1, sh.m - 2 + fs, sm, kind);
+    return ns_columns<D, NT, ALL_TEAMS>(a, sh, j, 0, q1, sh.m - 2 + fs, sm, kind) ||
+           saddle_columns<D, NT>(a, sh, j, 0, q1, sm, kind);
 }
 
 // Lebesgue values of the columns of a chunk: eight lanes per column, each over every eighth node of
@@ -1730,8 +1822,13 @@ __device__ __forceinline__ void ns_lebesgue(const Shape& sh, int c0, int qk, con
 
 // A later chunk of columns with the stored factors.
 template <int D, int NT>
-__device__ __forceinline__ void ns_solve_chunk(const SolveArgs& a, const Shape& sh, int j, int c0,
+__device__ __forceinline__ bool ns_solve_chunk(const SolveArgs& a, const Shape& sh, int j, int c0,
                                                int qk, const NullSmem& sm) {
+    if (s_ns_saddle) {
+        const bool ok = saddle_columns<D, NT>(a, sh, j, c0, qk, sm, 0);
+        if (ok) ns_lebesgue<NT>(sh, c0, qk, sm);
+        return ok;
+    }
     const int n = sh.n, M = sh.M;
     const int icoef = ns_coef<D>(sh), fs = ns_bits(icoef);
 #pragma unroll 1
@@ -1745,6 +1842,7 @@ __device__ __forceinline__ void ns_solve_chunk(const SolveArgs& a, const Shape& 
     __syncthreads();
     ns_columns<D, NT, false>(a, sh, j, c0, qk, sh.m - 2 + fs, sm, 0);
     ns_lebesgue<NT>(sh, c0, qk, sm);
+    return true;
 }
 
 // Weight of stencil position r in column c0 + c, column c of the chunk held in shared memory.
@@ -1760,11 +1858,6 @@ template <> struct SmemType<kNull> { using T = NullSmem; };
 template <int LAY> using SmemOf = typename SmemType<LAY>::T;
 
 // ------------------------------------------------------------------ traversal state machine
-// Acquire-release fence at device scope: orders this thread's earlier memory operations, and
-// those of its CTA that a barrier made visible to it, before its later ones, as seen by every
-// thread of the device.  Only threads that publish (or consume) traversal state execute it.
-__device__ __forceinline__ void fence_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
-
 __device__ __forceinline__ void push_center(const SolveArgs& a, int k) {
     fence_gpu();
     const int slot = atomicAdd(&a.ctr->q_tail, 1);
@@ -2005,7 +2098,7 @@ __global__ void __launch_bounds__(NT, min_blocks(LAY, NT)) k_traversal(SolveArgs
                 __syncthreads();  // sm.X is read until here
                 // (the shape is read again rather than kept in registers)
                 if (ok) {
-                    if constexpr (LAY == kNull) ns_solve_chunk<D, NT>(a, shape_of<D>(a, sbasis, j), j, c0, qk, sm);
+                    if constexpr (LAY == kNull) ok = ns_solve_chunk<D, NT>(a, shape_of<D>(a, sbasis, j), j, c0, qk, sm);
                     else solve_chunk<D, NT>(a, shape_of<D>(a, sbasis, j), c0, qk, sm, j, s_ref);
                 }
                 __syncthreads();
@@ -2057,13 +2150,6 @@ __global__ void __launch_bounds__(NT, min_blocks(LAY, NT)) k_traversal(SolveArgs
         }
         __syncthreads();
     }
-}
-
-// Normal-derivative right-hand side of node i's own stencil, replacing column 0 of the
-// right-hand-side block (unknowns in index order, before the factorization).
-template <int D, int NT>
-__device__ void neumann_rhs(const SolveArgs& a, const Shape& sh, int i, const StencilSmem& sm) {
-    for (int j = threadIdx.x; j < sh.n + sh.M; j += NT) sm.X[j * sm.xs] = neumann_value<D>(a, sh, i, j, sm.xi);
 }
 
 // FALLBACK re-solves (one right-hand side each), one launch per stencil class: `cls` is the

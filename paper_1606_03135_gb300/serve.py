@@ -59,7 +59,8 @@ def estimate_bytes(N: int, d: int, n: int, delta: float, ell: int = None) -> int
     """Upper bound of the device bytes a uniform-stencil job holds at once: the plan's stencil
     arrays, the cell-grid scratch of its kNN step, and the traversal and CSR arrays of its
     assembly, with every retention ball bounded by the stencil size (one node at delta = 1),
-    plus 1 MB for alignment and small tables.  Plans of K = n + C(ell + d, d) >= 100 unknowns
+    plus 1 MB for alignment and small tables and the 8 MB of blocks for stencils that the null space
+    cannot solve.  Plans of K = n + C(ell + d, d) >= 100 unknowns
     refine ill-conditioned solves by default, and their assembly then keeps, per resident CTA,
     the full K x K system, its first solutions and the residual's partial sums: at most 5 times
     the CTA's shared-memory system, so under 200 MB on a 152-SM GB300 (228 KB of shared memory
@@ -69,7 +70,7 @@ def estimate_bytes(N: int, d: int, n: int, delta: float, ell: int = None) -> int
     plan = N * (d * 8 + n * 4 + 8 + 4 + 4 + 8) + (2 * N + 64) * 12 + N * (8 + 8 * d)
     asm = N * (4 * 6 + 2 + n * 12 + 16) + N * ball * (n * 8 + 9)
     refined = ell is None or n + math.comb(ell + d, d) >= 100
-    return int(plan + asm + (1 << 20) + ((200 << 20) if refined else 0))
+    return int(plan + asm + (9 << 20) + ((200 << 20) if refined else 0))
 
 
 class Budget:

@@ -194,7 +194,8 @@ typedef struct {
  * bytes (LU option: 8 K (K + q + 4)) must fit the device's per-block limit (227 KB on GB300).
  * LU carries every column (q = the largest retention ball); LDL^T carries opts->rhs_chunk
  * columns and solves the rest in chunks of that many, so its limit is q = 1: in 3D,
- * n = 128 with degree 7 (K = 248) is too large.  Else RBFFD_EINVAL.  Errors: RBFFD_EINVAL,
+ * n = 128 with degree 7 (K = 248) is too large.  Else RBFFD_EINVAL.  Nodes have to be finite,
+ * with a bounding box whose squared diagonal is, else RBFFD_EINVAL.  Errors: RBFFD_EINVAL,
  * RBFFD_EDUPLICATE, RBFFD_ENOMEM, RBFFD_ECUDA.  On error *out is NULL and nothing leaks. */
 int rbffd_plan(const double* nodes, int64_t N, int d, int n, int ell, int m, double delta,
                const rbffd_opts* opts, void* stream, rbffd_plan_t* out);
@@ -288,7 +289,8 @@ int rbffd_export_lambda(rbffd_plan_t plan, double* lam_row, uint8_t* is_center);
  * share the array, so calls that overlap on the GPU (other streams, other host threads) race
  * and must be serialised by the caller; each call clears the status it reads.  Every call
  * ends by copying the device status to the host and waiting for `stream`
- * (RBFFD_EDUPLICATE for coincident nodes), so no call can be made while `stream` is being
+ * (RBFFD_EDUPLICATE for coincident nodes, RBFFD_EINVAL for nodes that are not finite or too far
+ * apart, as rbffd_plan), so no call can be made while `stream` is being
  * captured into a CUDA graph. */
 #define RBFFD_NOALLOC_MAX_NODES 32768
 int rbffd_stencils_noalloc(const double* nodes, int64_t N, int d, int n, double delta,

@@ -94,14 +94,31 @@ __device__ __forceinline__ double ord_val(unsigned long long k) {
 }
 
 // Cell size for about 2 nodes per cell and the first search ring, from the bounding box.
+// Nodes that are not finite, or so far apart that the square of the box's diagonal is not, are an
+// error: their distances have no order, and the search would not find n of them.  The grid is then
+// a single cell (indices stay in range), and no search runs on it (r0 = 0).
 template <int D>
 __device__ void set_grid_params(const double* L, const double* H, int N, int n, int ncell_max,
-                                GridParams* gp) {
+                                GridParams* gp, DevCounters* ctr) {
     double ext[3] = {0.0, 0.0, 0.0};
-    double vol = 1.0, maxext = 0.0;
+    double vol = 1.0, maxext = 0.0, diag2 = 0.0;
     for (int a = 0; a < D; ++a) {
         ext[a] = H[a] - L[a];
         maxext = fmax(maxext, ext[a]);
+        diag2 += ext[a] * ext[a];
+    }
+    if (!(diag2 < __longlong_as_double(0x7ff0000000000000LL))) {  // (NaN too)
+        set_error(ctr, RBFFD_EINVAL);
+        for (int a = 0; a < 3; ++a) {
+            gp->lo[a] = 0.0;
+            gp->dims[a] = 1;
+        }
+        gp->h = 1.0;
+        gp->inv_h = 0.0;
+        gp->ncell = 1;
+        gp->r0 = 0;
+        gp->xerr = 0.0f;
+        return;
     }
     if (!(maxext > 0.0)) maxext = 1.0;
     for (int a = 0; a < D; ++a) vol *= fmax(ext[a], 1e-3 * maxext);
@@ -145,7 +162,7 @@ __device__ void set_grid_params(const double* L, const double* H, int N, int n, 
 template <int D>
 __global__ void __launch_bounds__(256) k_grid_params(const double* __restrict__ X, int N, int n,
                                                      int ncell_max, BBoxAcc* acc,
-                                                     GridParams* gp) {
+                                                     GridParams* gp, DevCounters* ctr) {
     __shared__ unsigned long long s_lo[3][8], s_hi[3][8];
     __shared__ bool s_last;
     unsigned long long lo[3] = {~0ull, ~0ull, ~0ull}, hi[3] = {0ull, 0ull, 0ull};
@@ -187,7 +204,7 @@ __global__ void __launch_bounds__(256) k_grid_params(const double* __restrict__ 
         L[a] = ord_val(~*((volatile unsigned long long*)&acc->nlo[a]));
         H[a] = ord_val(*((volatile unsigned long long*)&acc->hi[a]));
     }
-    set_grid_params<D>(L, H, N, n, ncell_max, gp);
+    set_grid_params<D>(L, H, N, n, ncell_max, gp, ctr);
 }
 
 template <int D>
@@ -546,6 +563,14 @@ __global__ void __launch_bounds__(256) k_knn(const double* __restrict__ X, int N
     const GridParams g = *gp;
 
     for (int q = blockIdx.x * wpb + wib; q < N; q += gridDim.x * wpb) {
+        if (g.r0 == 0) {  // (an error is set: only keep the indices in range)
+            for (int t = lane; t < n; t += 32) nbr[(size_t)q * n + t] = q;
+            if (lane == 0) {
+                rho2[q] = 0.0;
+                ball_len[q] = 1;
+            }
+            continue;
+        }
         double xq[3];
         float xqf[3];
         int c0[3];
@@ -801,7 +826,7 @@ static int grid_and_knn(const double* X, int N, int n, double omd2, void* scratc
     int dev = 0, sms = 1;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    k_grid_params<D><<<nb < sms ? nb : sms, tb, 0, s>>>(X, N, n, ncell_max, acc, gp);
+    k_grid_params<D><<<nb < sms ? nb : sms, tb, 0, s>>>(X, N, n, ncell_max, acc, gp, ctr);
     k_cell_count<D><<<nb, tb, 0, s>>>(X, N, gp, cell_of, count, rank);
     k_scan<int><<<1, 1024, 0, s>>>(count, start, ncell_max, &gp->ncell);
     k_cell_fill<D><<<nb, tb, 0, s>>>(X, N, cell_of, start, rank, sorted_idx, sorted_X,

@@ -981,9 +981,7 @@ __device__ __forceinline__ void lebesgue_values(int n, int K, int q, const Stenc
 // at y = 0 is -m ||xi_u||^(m-2) (xi_u . n), and of the monomials only the linear ones have a
 // nonzero gradient there (d/dn xi_a = n_a).
 template <int D>
-__device__ __forceinline__ double neumann_at(const SolveArgs& a, const Shape& sh, int i, int u,
-                                             const double* xj) {
-    const double* nv = a.nrm + (size_t)i * D;
+__device__ __forceinline__ double neumann_at(const Shape& sh, const double* nv, int u, const double* xj) {
     if (u < sh.n) {
         const double mm = exact_double(sh.m);
         double r2 = xj[0] * xj[0], dot = xj[0] * nv[0];
@@ -999,16 +997,33 @@ __device__ __forceinline__ double neumann_at(const SolveArgs& a, const Shape& sh
     return (l > 0 && sh.bs.parent[l] == 0) ? nv[sh.bs.var[l]] : 0.0;
 }
 template <int D>
-__device__ __forceinline__ double neumann_value(const SolveArgs& a, const Shape& sh, int i, int u,
-                                                const double* xi) {
-    return neumann_at<D>(a, sh, i, u, xi + (u < sh.n ? u * D : 0));
+__device__ __forceinline__ double neumann_value(const Shape& sh, const double* nv, int u, const double* xi) {
+    return neumann_at<D>(sh, nv, u, xi + (u < sh.n ? u * D : 0));
+}
+
+// Normals of any length: the null-space solves hold right-hand sides in units fixed by the exponent,
+// so they take the normal times 2^-e, its largest component in (1/2, 1] (unit vectors, in 2D and 3D:
+// e = 0), and the row is scaled back at the end.  Returns e (0 for a zero normal).
+template <int D>
+__device__ __forceinline__ int scaled_normal(const SolveArgs& a, int i, double* nv) {
+    double top = 0.0;
+    for (int c = 0; c < D; ++c) {
+        nv[c] = a.nrm[(size_t)i * D + c];
+        top = fmax(top, fabs(nv[c]));
+    }
+    int e = 0;
+    const double m = frexp(top, &e);  // in [1/2, 1)
+    if (m == 0.5) --e;
+    if (top == 0.0) e = 0;
+    for (int c = 0; c < D; ++c) nv[c] = scalbn(nv[c], -e);
+    return e;
 }
 
 // Normal-derivative right-hand side of node i's own stencil, replacing column 0 of the
 // right-hand-side block (unknowns in index order, before the factorization).
 template <int D, int NT>
-__device__ void neumann_rhs(const SolveArgs& a, const Shape& sh, int i, const StencilSmem& sm) {
-    for (int j = threadIdx.x; j < sh.n + sh.M; j += NT) sm.X[j * sm.xs] = neumann_value<D>(a, sh, i, j, sm.xi);
+__device__ void neumann_rhs(const Shape& sh, const double* nv, const StencilSmem& sm) {
+    for (int j = threadIdx.x; j < sh.n + sh.M; j += NT) sm.X[j * sm.xs] = neumann_value<D>(sh, nv, j, sm.xi);
 }
 
 // Team sizes whose traversal kernels carry the refinement step: the 96- and 128-thread teams
@@ -1076,7 +1091,7 @@ __device__ void refine_columns(const SolveArgs& a, const Shape& sh, int c0, int 
         gX0[sm.perm[r] * qk + c] = sm.X[r * xs + c];
     }
     if (kind == 2) {
-        for (int r = tid; r < K; r += NT) sm.X[r * xs] = neumann_value<D>(a, sh, i, sm.perm[r], sm.xi);
+        for (int r = tid; r < K; r += NT) sm.X[r * xs] = neumann_value<D>(sh, a.nrm + (size_t)i * D, sm.perm[r], sm.xi);
     } else {
         chunk_rhs<D, NT>(sh, c0, qk, sm, a.fma_r2 != 0);
     }
@@ -1324,8 +1339,10 @@ __device__ void ns_constraints_fixed(const SolveArgs& a, const Shape& sh, int j,
         const int c = small_div(e, M), l = e - c * M;
         long long v = 0;
         if (kind == 2) {
+            double nv[D];
             const double x0[D] = {};
-            v = to_fixed(neumann_at<D>(a, sh, j, n + l, x0), gs - kTabBits);
+            scaled_normal<D>(a, j, nv);
+            v = to_fixed(neumann_at<D>(sh, nv, n + l, x0), gs - kTabBits);
         } else {
             const long long* row = T + sm.cols[c] * ldm;
             for (int d = 0; d < D; ++d) {
@@ -1365,8 +1382,10 @@ __device__ void ns_constraints(const SolveArgs& a, const Shape& sh, int j, int q
         const int c = e / M, l = e - c * M;
         double v = 0.0;
         if (kind == 2) {
+            double nv[D];
             const double x0[D] = {};
-            v = neumann_at<D>(a, sh, j, n + l, x0);
+            scaled_normal<D>(a, j, nv);
+            v = neumann_at<D>(sh, nv, n + l, x0);
         } else {
             const double* row = sm.T + sm.cols[c] * ldm;
             for (int d = 0; d < D; ++d) {
@@ -1595,7 +1614,9 @@ __device__ __noinline__ void ns_refine(const SolveArgs& a, const Shape& sh, int 
         const int c = 4 * g + l4;  // lane l4 adds f of the group's column l4
         double f = l4 == 0 ? r[0] : (l4 == 1 ? r[1] : (l4 == 2 ? r[2] : r[3]));
         if (kind == 2) {
-            f += neumann_at<D>(a, sh, j, 0, x);
+            double nv[D];
+            scaled_normal<D>(a, j, nv);
+            f += neumann_at<D>(sh, nv, 0, x);
         } else if (sm.order[p] != sm.cols[c0 + c]) {
             double y[D];
             const int t = sm.pos[sm.cols[c0 + c]];
@@ -1699,7 +1720,9 @@ __device__ __noinline__ bool saddle_columns(const SolveArgs& a, const Shape& sh,
         if (b == 0) {
             assemble_local<D, true, NT>(a, sh, j, q, st);
             if (kind == 2) {
-                neumann_rhs<D, NT>(a, sh, j, st);
+                double nv[D];
+                scaled_normal<D>(a, j, nv);
+                neumann_rhs<D, NT>(sh, nv, st);
                 __syncthreads();
             }
             ok = factor_solve_ldlt<NT>(K, q, st);
@@ -1792,11 +1815,13 @@ __device__ bool ns_solve(const SolveArgs& a, const Shape& sh, int j, int q, int 
     ns_pairs<D, NT>(sh, q1, icoef, fs, sm);
     __syncthreads();
     if (kind == 2) {
+        double nv[D];
+        scaled_normal<D>(a, j, nv);
 #pragma unroll 1
         for (int u = tid; u < n; u += NT) {
             const int p = sm.pos[u];
             fixed(sm.X)[p < M ? p : sm.x2 + p - M] =
-                to_fixed(neumann_at<D>(a, sh, j, u, sm.xi + u * D), p < M ? sh.m + sm.eg[0] + kSumUnit - 1 : sh.m - 2 + fs - kPowerBits);
+                to_fixed(neumann_at<D>(sh, nv, u, sm.xi + u * D), p < M ? sh.m + sm.eg[0] + kSumUnit - 1 : sh.m - 2 + fs - kPowerBits);
         }
         __syncthreads();
     }
@@ -2186,7 +2211,7 @@ __global__ void __launch_bounds__(NT, min_blocks(LAY, NT)) k_fallback_solve(Solv
         if constexpr (LAY != kNull) {
             assemble_local<D, LAY == kPacked, NT>(a, sh, i, 1, sm);
             if (kind == 2) {
-                neumann_rhs<D, NT>(a, sh, i, sm);
+                neumann_rhs<D, NT>(sh, a.nrm + (size_t)i * D, sm);
                 __syncthreads();
             }
         }
@@ -2209,10 +2234,15 @@ __global__ void __launch_bounds__(NT, min_blocks(LAY, NT)) k_fallback_solve(Solv
         if (__double_as_longlong(r2c) <= 0) r2c = 1.0;
         // weights of the scaled problem times rho^-2 (Laplacian) or rho^-1 (normal derivative)
         const double scale = kind == 2 ? rcp_fixed(sqrt(r2c)) : rcp_fixed(r2c);
+        int en = 0;
+        if constexpr (LAY == kNull) {
+            double nv[D];
+            if (kind == 2) en = scaled_normal<D>(a, i, nv);
+        }
         for (int r = tid; r < sh.n; r += NT)
-            a.slot_w[slot * a.n + r] = ok ? weight(sh, r, 0, 0, sm) * scale : nan;
+            a.slot_w[slot * a.n + r] = ok ? scalbn(weight(sh, r, 0, 0, sm), en) * scale : nan;
         if (tid == 0) {
-            a.slot_lam[slot] = ok ? sm.lam[0] : nan;
+            a.slot_lam[slot] = ok ? scalbn(sm.lam[0], en) : nan;
             if (!ok) {
                 atomicAdd(&a.ctr->n_singular, 1);
                 set_error(a.ctr, RBFFD_ESINGULAR);

@@ -17,9 +17,9 @@
 // (measured: 2.0 and 62.6).  In this form two thirds of the work are the two matrix products,
 // which run on the integer pipe in fixed point: operands are 59-bit integers in two limbs
 // (v = hi 2^28 + lo, |lo| <= 2^27) scaled by a power of two per matrix, a product is three
-// multiply-adds (hi hi, hi lo + lo hi; lo lo, below 2^-62 of the scale, only where S is formed) and
-// the sums are exact,
-// so the cancellation of S (entries near 0.1 out of sums near 100) costs nothing.
+// multiply-adds (hi hi, hi lo + lo hi; lo lo is below 2^-62 of the scale) and the sums are exact.
+// A is that of r^m less a polynomial (KernelUnits in traversal.cuh), which S does not see and which
+// makes its entries, and with them the units, up to 23 times smaller.
 #pragma once
 
 #include "fp64_int.cuh"
@@ -30,11 +30,11 @@ namespace rbffd {
 // ------------------------------------------------------------------ fixed point
 constexpr int kFixBits = 58;   // |v| < 2^58 for an operand below its scale 2^e: v = x 2^(58 - e)
 constexpr int kLimbBits = 28;
-constexpr int kPowerBits = 62;  // of the powers of r and of f, which are not operands of products
+constexpr int kPowerBits = 62;  // of phi and of f, which are not operands of products
 
 // The conversions and dot products below that are used in several places are functions of their
 // own, loops are not unrolled beyond what hides their latency, and quotients of small integers take
-// an FP32 reciprocal: the kernels run the phases of up to 28 systems side by side on an SM, and with
+// an FP32 reciprocal: the kernels run the phases of up to 22 systems side by side on an SM, and with
 // everything inlined (218 KB of code) waiting for instructions took a third of the time (3D ball,
 // N = 100,000, delta = 1: 16.7 ms, against 9.9 ms at 128 KB).
 
@@ -143,23 +143,6 @@ struct LimbSum {
     }
 };
 
-// The same with the products of the lower limbs, for the sums that S is formed of: without them
-// (0.1 units a term) its weights of one-sided degree-5 stencils are 2 to 20 times further off.
-struct FullSum : LimbSum {
-    long long l = 0;
-    __device__ __forceinline__ void mac(int2 x, int2 y) {
-        LimbSum::mac(x, y);
-        l += (long long)x.y * y.y;
-    }
-    __device__ __forceinline__ void fold() {
-        m += l >> kLimbBits;
-        l &= (1ll << kLimbBits) - 1;
-        LimbSum::fold();
-    }
-    __device__ __forceinline__ long long total() const {
-        return h + ((m + (l >> kLimbBits) + (1ll << (kLimbBits - 1))) >> kLimbBits);
-    }
-};
 constexpr int kSumUnit = 2 * kLimbBits - 2 * kFixBits;  // -60
 
 // ------------------------------------------------------------------ shared-memory layout
@@ -195,7 +178,7 @@ struct NullSmem {
                   //   (doubles), then the unscaled factor columns; may lie over A11
     double* X;    // one row of ldx words per column of the chunk: f1 (then f1 - A11 ghat / 2, its
                   //   limbs, the limbs of v), and from word x2 on f2 (then v, doubles)
-    double* xi;   // n x D scaled stencil coordinates
+    long long* xi;  // n x D scaled stencil coordinates (ns_coordinates)
     double* rd;   // s reciprocal pivots
     double* wb;   // s unscaled pivot column
     short* eg;    // qmax scale exponents of the ghat rows
@@ -244,7 +227,7 @@ __device__ __forceinline__ void carve_ns(char* p, int n, int M, int qcap, int qm
         sm.S = w;
         w += s * (s + 1) >> 1;
     }
-    sm.xi = w;
+    sm.xi = reinterpret_cast<long long*>(w);
     sm.rd = w;  // (the coordinates are done with when S is factored, unless later chunks need them)
     w += n * D;
     if (qcap < qmax) {
@@ -276,7 +259,6 @@ __device__ __forceinline__ long long* fixed(double* p) { return reinterpret_cast
 
 // ------------------------------------------------------------------ the constraints
 __shared__ int s_ns_ok, s_ns_eb, s_ns_ec;
-__shared__ int s_ns_l1;  // bits of a float: the largest row sum of |B|
 
 // A team's barrier.
 template <int NT>
@@ -608,7 +590,7 @@ __device__ void ns_product_c(int n, int M, int i0, int c0, int qk, int eA, const
         const int4* B = reinterpret_cast<const int4*>(sm.T + (M + i + c0) * ldm);
         const int4* A = reinterpret_cast<const int4*>(sm.T + j);
         const int lc = ldm >> 1, db = two_i ? lc : 0;
-        FullSum a0, a1, b0, b1;
+        LimbSum a0, a1, b0, b1;
 #pragma unroll 1
         for (int k = 0; 2 * k < M; ++k) {
             const int4 x = B[k], y = B[k + db], u = A[0], v = A[lc];
@@ -717,7 +699,7 @@ __device__ void ns_product_s(int n, int M, bool triangle, int c0, int qk, const 
         const int4* Cj = reinterpret_cast<const int4*>(sm.C + j * ldm);
         const int db = two_i ? ldm >> 1 : 0, dc = two_i ? (column ? sm.ldx : ldm) >> 1 : 0;
         const int dj = two_j ? ldm >> 1 : 0;
-        FullSum aa, ab, ba, bb;
+        LimbSum aa, ab, ba, bb;
 #pragma unroll 1
         for (int k = 0; 2 * k < M; ++k) {
             auto half_step = [&](int4 bi, int4 bk, int4 cj, int4 ck) {

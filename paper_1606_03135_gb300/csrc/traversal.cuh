@@ -1279,20 +1279,32 @@ __device__ __forceinline__ void lebesgue_values(int n, int K, int q, const Stenc
 
 // ------------------------------------------------------------------ null-space solves
 // Stencil coordinates (x - x_c) / rho_j, rounded to FP64 as everywhere (the quotient by a reciprocal
-// and one residual), and the identity order.
-template <int D, int NT>
-__device__ void ns_coordinates(const SolveArgs& a, const Shape& sh, int j, const NullSmem& sm) {
-    const int tid = threadIdx.x, n = sh.n;
+// and one residual).
+struct Radius { double rho, rcp; };
+__device__ __forceinline__ Radius ns_radius(const SolveArgs& a, int j) {
     double r2c = a.rho2[j];
     if (__double_as_longlong(r2c) <= 0) r2c = 1.0;
-    const double rho = sqrt_fast(r2c), rcp = rcp_fixed(rho);
+    const double rho = sqrt_fast(r2c);
+    return {rho, rcp_fixed(rho)};
+}
+template <int D>
+__device__ __forceinline__ double ns_coordinate(const SolveArgs& a, int j, int t, int c, const Radius& r) {
+    const int id = a.nbr[(size_t)j * a.n + t];
+    const double dx = __dsub_rn(a.X[(size_t)id * D + c], a.X[(size_t)j * D + c]);
+    const double x = dx * r.rcp;
+    return fma(fma(-x, r.rho, dx), r.rcp, x);
+}
+
+// All of them in units of 2^-kCoordBits (which holds every bit of a coordinate of 2^-8 and more), and
+// the identity order.
+constexpr int kCoordBits = 61;
+template <int D, int NT>
+__device__ void ns_coordinates(const SolveArgs& a, const Shape& sh, int j, const NullSmem& sm) {
+    const Radius r = ns_radius(a, j);
 #pragma unroll 1
-    for (int e = tid; e < n * D; e += NT) {
+    for (int e = threadIdx.x; e < sh.n * D; e += NT) {
         const int t = e / D, c = e - t * D;
-        const int id = a.nbr[(size_t)j * a.n + t];
-        const double dx = __dsub_rn(a.X[(size_t)id * D + c], a.X[(size_t)j * D + c]);
-        const double x = dx * rcp;
-        sm.xi[e] = fma(fma(-x, rho, dx), rcp, x);
+        sm.xi[e] = to_fixed(ns_coordinate<D>(a, j, t, c, r), -kCoordBits);
         if (c == 0) sm.order[t] = t;
     }
 }
@@ -1321,7 +1333,7 @@ __device__ void ns_constraints_fixed(const SolveArgs& a, const Shape& sh, int j,
     for (int t = tid; t < n; t += NT) {  // each monomial = an earlier one times one coordinate
         int2 x[D];
 #pragma unroll
-        for (int c = 0; c < D; ++c) x[c] = split_limbs(to_fixed(sm.xi[t * D + c], -kTabBits));
+        for (int c = 0; c < D; ++c) x[c] = split_limbs(shift_right(sm.xi[t * D + c], kCoordBits - kTabBits));
         long long* row = T + t * ldm;
         row[0] = 1ll << kTabBits;
 #pragma unroll 1
@@ -1363,10 +1375,11 @@ __device__ void ns_constraints(const SolveArgs& a, const Shape& sh, int j, int q
     const int tid = threadIdx.x;
     const int n = sh.n, M = sh.M, ldm = sm.ldm;
     const Basis& bs = sh.bs;
+    const Radius r = ns_radius(a, j);
 #pragma unroll 1
     for (int t = tid; t < n; t += NT) {
         double x[D];
-        for (int c = 0; c < D; ++c) x[c] = sm.xi[t * D + c];
+        for (int c = 0; c < D; ++c) x[c] = ns_coordinate<D>(a, j, t, c, r);
         double* row = sm.T + t * ldm;
         row[0] = 1.0;
 #pragma unroll 1
@@ -1411,46 +1424,113 @@ __device__ __noinline__ bool ns_eliminate_fp64(const SolveArgs& a, const Shape& 
     return true;
 }
 
-// r^(m-2) and r^m of two stencil nodes as fractions of 2^(m-2) and 2^m with kPowerBits bits (the
-// powers of near nodes, whose differences make the small eigenvalues of S, would lose with fewer
-// against the relative precision of FP64).  The squared
-// distance is formed in FP64 without FMA, rounded as the oracle's (8 instructions in 3D; formed in
-// fixed point it took 48 others and made the weights two to five times closer to an exact solve, but
-// further from any FP64 one); its root and the powers of u = r / 2 <= 1 (the stencil's radius is 1)
-// in fixed point.
+// The kernel.  A polynomial p of degree m - 1 in r changes A by P Y^T + Y P^T and so neither S nor the
+// weights (2 ell + 1 >= m), as long as the same p is taken off f.  The solves use
+//   phi(r) = r^m - p(r^2) = 2^m z^((m-1)/2) (u - beta),   u = r / 2, z = u^2 (r <= 2: the radius is 1)
+// with the beta that makes |phi| small: 9, 16 and 23 times below 2^m for m = 3, 5, 7.  S is formed of
+// entries of that size, and the grids of A, C and its sums are as much finer.  With r^m itself their
+// rounding was as large as the squared distances' in 2D.  Median errors over 120 rows against an
+// 80-bit solve (r^7, this / r^m itself / the saddle-point layout): disk, degree 3, n = 21, 2.3e-13 /
+// 3.1e-13 / 2.3e-13; degree 4, n = 31, 1.6e-12 / 2.4e-12 / 1.8e-12; lattice, degree 4, 3.9e-13 /
+// 1.5e-12 / 4.0e-13; ball, degree 4, n = 71, 2.2e-12 / 2.4e-12 / 2.5e-12; degree 5, n = 113, 1.2e-11 /
+// 1.5e-11 / 1.3e-11.  It costs 30 instructions a pair and saves the products of lower limbs that the
+// sums needed before (552 plans: the same time, geometric mean of the ratios 1.00).
+struct KernelUnits {
+    int beta;    // of 256
+    int eA, eF;  // |phi| < 2^eA, |f| < 2^eF
+    int fs;      // eF = m - 2 + fs
+    int c1, c3;  // f = 2^(m-2) (c1 u z^k - beta c3 z^k), k = (m - 3) / 2: the Laplacian's factors, or
+                 // (kind 2) those of the derivative against -(x . n)
+};
+
 template <int D>
-__device__ __noinline__ void ns_powers(const double* xa, const double* xb, int m, long long* pm2,
-                                       long long* pm) {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(sqdist_rn<D>(xa, xb));
-    const int e = (int)(b >> 52) - 1023, odd = e & 1;  // r^2 = m 4^h, m in [1, 4)
-    const unsigned long long N = ((b & 0xFFFFFFFFFFFFFull) | (1ull << 52)) << (10 + odd);  // m 2^62
-    const unsigned long long z = N >> min(2 + odd - e, 63) << 1;  // (r / 2)^2 2^63
-    unsigned long long u = ((unsigned long long)sqrt_core(N) << 2) >> min(1 - ((e - odd) >> 1), 63);
+__device__ __forceinline__ KernelUnits ns_units(int m, int kind) {
+    KernelUnits k;
+    k.beta = m == 3 ? 229 : (m == 5 ? 242 : 245);
+    k.eA = m == 3 ? 0 : m - 4;
+    k.fs = kind == 2 ? 1 : (m == 3 ? 3 : 4);
+    k.eF = m - 2 + k.fs;
+    k.c1 = kind == 2 ? m : m * (m + D - 2);
+    k.c3 = kind == 2 ? m - 1 : (m - 1) * (m + D - 3);
+    return k;
+}
+
+// What phi and f of a pair are made of: phi in 2^-62 of 2^m, pk = z^k (u - beta) in 2^-62, z in 2^-63,
+// and delta, below.
+struct PairPowers {
+    long long phi, pk, z;
+    int delta;
+};
+
+// The squared distance in u is formed in FP64 without FMA, rounded as the oracle's: the weights are as
+// far from an exact solve as that rounding puts every FP64 solver's, and so near to theirs.  In p it
+// has to be exact, or p would be no polynomial: z and the exact square differ by delta in 2^-63, a
+// dozen bits, found from the low words of the coordinates' integer differences.  The root and the
+// powers are fixed point.
+template <int D>
+__device__ __noinline__ PairPowers ns_powers(const long long* xa, const long long* xb, int m, int beta) {
+    double r2 = 0.0;
+    unsigned H = 0u;
+    long long mid = 0;
+    unsigned long long low = 0;
+#pragma unroll
+    for (int c = 0; c < D; ++c) {
+        const long long d = xa[c] - xb[c];  // (the sum of d^2 is 2^(2 kCoordBits) r^2 = 2^124 z)
+        const double t = __ll2double_rn(d);
+        r2 = c == 0 ? __dmul_rn(t, t) : __dadd_rn(r2, __dmul_rn(t, t));
+        const int hi = (int)((d + (1ll << 31)) >> 32), lo = (int)d;
+        H += (unsigned)(hi * hi);
+        mid += (long long)hi * lo;
+        low += (unsigned long long)((long long)lo * lo);
+    }
+    const unsigned exact = (H << 3) + (unsigned)(mid >> 28) + (unsigned)(low >> 61);  // 2^63 z, low word
+    const unsigned long long b = (unsigned long long)__double_as_longlong(r2);
+    const int e = (int)(b >> 52) - 1023 - 2 * kCoordBits, odd = e & 1;  // r^2 = w 4^h, w in [1, 4)
+    const unsigned long long N = ((b & 0xFFFFFFFFFFFFFull) | (1ull << 52)) << (10 + odd);  // w 2^62
+    const unsigned long long zr = b == 0ull ? 0ull : N >> min(2 + odd - e, 63) << 1;
+    PairPowers o;
+    o.delta = (int)((unsigned)zr - exact);
+    o.z = (long long)min(zr, 0x7fffffffffffffffull);
+    const unsigned long long u =
+        b == 0ull ? 0ull : ((unsigned long long)sqrt_core(N) << 2) >> min(1 - ((e - odd) >> 1), 63);
+    long long p = (long long)u - ((long long)beta << (kPowerBits - 8));
+    const int k = (m - 3) / 2;
 #pragma unroll 1
-    for (int s = 0; s < (m - 3) / 2; ++s) u = __umul64hi(u << 1, z);
-    *pm2 = (long long)u;
-    *pm = (long long)__umul64hi(u << 1, z);
+    for (int s = 0; s < k; ++s) p = __mul64hi(p << 1, o.z);
+    o.pk = p;
+    // beta (z^(k+1) - its exact value) = beta (k + 1) z^k delta, z^k with 12 bits
+    const int zt = (int)(o.z >> 51), zk = k == 0 ? 4096 : (k == 1 ? zt : zt * zt >> 12);
+    o.phi = __mul64hi(p << 1, o.z) + ((long long)o.delta * (beta * (k + 1) * zk) >> 21);
+    return o;
 }
 
-// coef r^(m-2) as a fraction of 2^(m-2+fs) with kPowerBits bits, coef <= 2^fs.
-__device__ __forceinline__ long long ns_rhs_fixed(long long pm2, int coef, int fs) {
-    return (((pm2 >> 32) * coef) << (32 - fs)) + (((pm2 & 0xffffffffll) * coef) >> fs);
+// v c 2^-s, 0 <= c < 2^20, s <= 32.
+__device__ __forceinline__ long long scale_by(long long v, int c, int s) {
+    return (((v >> 32) * c) << (32 - s)) + (((v & 0xffffffffll) * c) >> s);
 }
 
-// Scale of the columns' f rows: Laplacians reach coef 2^(m-2) (coef = m (m + D - 2) <= 2^fs), normal
-// derivatives m.
-template <int D>
-__device__ __forceinline__ int ns_coef(const Shape& sh) { return sh.m * (sh.m + D - 2); }
-__device__ __forceinline__ int ns_bits(int v) { return 32 - __clz(v - 1); }  // v <= 2^bits
+// f of a pair, in 2^(eF - kPowerBits): c1 u z^k - beta c3 z^k = c1 pk + beta (c1 - c3) z^k, and as above
+// for the exact z^k of p.
+__device__ __forceinline__ long long ns_rhs_fixed(const PairPowers& o, int m, const KernelUnits& ku) {
+    const long long zk = m == 3 ? 1ll << kPowerBits : (m == 5 ? o.z >> 1 : __mul64hi(o.z, o.z));
+    const int zt = (int)(o.z >> 51), dz = m == 3 ? 0 : (m == 5 ? 4096 : 2 * zt);  // k z^(k-1)
+    const long long fix = (long long)o.delta * (ku.beta * ku.c3) * dz >> 21;
+    return scale_by(o.pk, ku.c1, ku.fs) + scale_by(zk, (ku.c1 - ku.c3) * ku.beta, ku.fs + 8) + (fix >> ku.fs);
+}
+
+// From f's unit to that of f1 in a column of scale 2^eg.
+__device__ __forceinline__ int ns_f1_shift(const KernelUnits& ku, int eg) {
+    return ku.eF - kPowerBits - (ku.eA + eg + kSumUnit - 1);
+}
 
 // A11 (limbs, over the eliminated rows of the tableau), A21 (in C) and what the columns' f share
 // with them: the pairs of tableau rows with at least one basic node, (i, j) with j < M and i > j,
 // flattened by columns; f's entries at the other nodes of a column whose node is not basic either
-// start from zero (ns_finish adds them with A22).  A21 and f1 count 2^(m + scale of the row - 61) (the
-// unit of ns_product_c), f2 2^(m - 2 + fs - 62).  In integers throughout: about 200 issue slots
-// per warp and pair, where the FP64 form has 14 FP64 instructions of 64 cycles each.
+// start from zero (ns_finish adds them with A22).  A21 and f1 count 2^(eA + scale of the row - 61) (the
+// unit of ns_product_c), f2 2^(eF - 62).  In integers but for the squared distance: about 230 issue
+// slots per warp and pair, where the FP64 form has 14 FP64 instructions of 64 cycles each.
 template <int D, int NT>
-__device__ void ns_pairs(const Shape& sh, int q, int icoef, int fs, const NullSmem& sm) {
+__device__ void ns_pairs(const Shape& sh, int q, const KernelUnits& ku, const NullSmem& sm) {
     const int tid = threadIdx.x;
     const int n = sh.n, M = sh.M, m = sh.m, ldm = sm.ldm, s = n - M, eB = s_ns_eb;
     const int rect = s * M, total = rect + (M >> 1) * M;
@@ -1468,36 +1548,38 @@ __device__ void ns_pairs(const Shape& sh, int q, int icoef, int fs, const NullSm
             j = low ? o : o - p - 1;
         }
         const int ra = sm.order[i], rb = sm.order[j];
-        long long pm2, pm;
-        ns_powers<D>(sm.xi + ra * D, sm.xi + rb * D, m, &pm2, &pm);
+        const PairPowers o = ns_powers<D>(sm.xi + ra * D, sm.xi + rb * D, m, ku.beta);
         if (i < M) {
-            const int2 v = split_limbs(shift_right(pm, kPowerBits - kFixBits));
+            const int2 v = split_limbs(shift_fixed(o.phi, m - ku.eA - (kPowerBits - kFixBits)));
             *limbs(sm.T + i * ldm + j) = v;
             *limbs(sm.T + j * ldm + i) = v;
         } else {
-            fixed(sm.C)[(i - M) * ldm + j] = shift_fixed(pm, 3 - eB - (kPowerBits - kFixBits));
+            fixed(sm.C)[(i - M) * ldm + j] = shift_fixed(o.phi, m - kPowerBits - (ku.eA + eB + kSumUnit - 1));
         }
         const int ca = sm.colof[ra], cb = sm.colof[rb];
         if ((ca >= 0 && ca < q) || (cb >= 0 && cb < q)) {
-            const long long f = ns_rhs_fixed(pm2, icoef, fs);
+            const long long f = ns_rhs_fixed(o, m, ku);
 #pragma unroll 1
             for (int k = 0; k < 2; ++k) {  // f of column c at row r
                 const int c = k ? cb : ca, r = k ? i : j;
                 if (c < 0 || c >= q) continue;
-                fixed(sm.X)[c * sm.ldx + (r < M ? r : sm.x2 + r - M)] = r < M ? shift_fixed(f, fs - 3 - sm.eg[c]) : f;
+                fixed(sm.X)[c * sm.ldx + (r < M ? r : sm.x2 + r - M)] = r < M ? shift_fixed(f, ns_f1_shift(ku, sm.eg[c])) : f;
             }
         }
     }
 #pragma unroll 1
-    for (int t = tid; t < n; t += NT) {  // r = 0
+    for (int t = tid; t < n; t += NT) {  // r = 0: phi = 0, and f = 0 but at r^3
         const int p = sm.pos[t], c = sm.colof[t];
         if (p < M) sm.T[p * ldm + p] = 0.0;
         if (c >= 0 && c < q) {
-            double* X = sm.X + c * sm.ldx;
-            if (p < M) X[p] = 0.0;
-            else
+            long long* X = fixed(sm.X) + c * sm.ldx;
+            const long long f = ns_rhs_fixed(ns_powers<D>(sm.xi + t * D, sm.xi + t * D, m, ku.beta), m, ku);
+            if (p < M) {
+                X[p] = shift_fixed(f, ns_f1_shift(ku, sm.eg[c]));
+            } else {
 #pragma unroll 1
-                for (int i = 0; i < s; ++i) X[sm.x2 + i] = 0.0;
+                for (int i = 0; i < s; ++i) X[sm.x2 + i] = i == p - M ? f : 0;
+            }
         }
     }
 }
@@ -1506,8 +1588,8 @@ __device__ void ns_pairs(const Shape& sh, int q, int icoef, int fs, const NullSm
 // nodes that are not basic; columns a and s - 1 - a of the triangle together have s + 1 entries), and
 // S becomes doubles.
 template <int D, int NT>
-__device__ void ns_finish(const Shape& sh, int qk, int icoef, int fs, int kind, const NullSmem& sm) {
-    const int n = sh.n, M = sh.M, s = n - M, eA = sh.m, eB = s_ns_eb, eC = s_ns_ec;
+__device__ void ns_finish(const Shape& sh, int qk, const KernelUnits& ku, int kind, const NullSmem& sm) {
+    const int n = sh.n, M = sh.M, s = n - M, m = sh.m, eB = s_ns_eb, eC = s_ns_ec;
     const int unit = eB + eC + kSumUnit, half = (s + 1) >> 1;
 #pragma unroll 1
     for (int e = threadIdx.x; e < half * (s + 1); e += NT) {
@@ -1519,13 +1601,12 @@ __device__ void ns_finish(const Shape& sh, int qk, int icoef, int fs, int kind, 
         long long a22 = 0;
         if (i != j) {
             const int ra = sm.order[M + i], rb = sm.order[M + j];
-            long long pm2, pm;
-            ns_powers<D>(sm.xi + ra * D, sm.xi + rb * D, sh.m, &pm2, &pm);
-            a22 = shift_fixed(pm, eA - kPowerBits - unit);
+            const PairPowers o = ns_powers<D>(sm.xi + ra * D, sm.xi + rb * D, m, ku.beta);
+            a22 = shift_fixed(o.phi, m - kPowerBits - unit);
             const int ca = sm.colof[ra], cb = sm.colof[rb];
             if (kind != 2 && ((ca >= 0 && ca < qk) || (cb >= 0 && cb < qk))) {
-                const long long f = ns_rhs_fixed(pm2, icoef, fs);
-                const int u = eA - 2 + fs - kPowerBits - kSumUnit - eC;  // of f, against 2^eg units
+                const long long f = ns_rhs_fixed(o, m, ku);
+                const int u = ku.eF - kPowerBits - kSumUnit - eC;  // of f, against 2^eg units
                 if (ca >= 0 && ca < qk) fixed(sm.X)[ca * sm.ldx + sm.x2 + j] += shift_fixed(f, u - sm.eg[ca]);
                 if (cb >= 0 && cb < qk) fixed(sm.X)[cb * sm.ldx + sm.x2 + i] += shift_fixed(f, u - sm.eg[cb]);
             }
@@ -1755,9 +1836,9 @@ __device__ __noinline__ bool saddle_columns(const SolveArgs& a, const Shape& sh,
 // The columns c0 .. c0+qk-1 from their f rows on (the triangle's products and factorization with
 // the first chunk).  f counts 2^(eF - kPowerBits).
 template <int D, int NT, bool ALL_TEAMS>
-__device__ bool ns_columns(const SolveArgs& a, const Shape& sh, int j, int c0, int qk, int eF,
+__device__ bool ns_columns(const SolveArgs& a, const Shape& sh, int j, int c0, int qk, const KernelUnits& ku,
                            const NullSmem& sm, int kind) {
-    const int n = sh.n, M = sh.M, s = n - M, eA = sh.m;
+    const int n = sh.n, M = sh.M, s = n - M, eA = ku.eA, eF = ku.eF;
     const bool first = c0 == 0;
     ns_product_c<NT>(n, M, first ? 0 : s, c0, qk, eA, sm);
     __syncthreads();
@@ -1769,7 +1850,7 @@ __device__ bool ns_columns(const SolveArgs& a, const Shape& sh, int j, int c0, i
     ns_product_s<NT>(n, M, first, c0, qk, sm);
     __syncthreads();
     if (first) {
-        ns_finish<D, NT>(sh, qk, ns_coef<D>(sh), eF - sh.m + 2, kind, sm);
+        ns_finish<D, NT>(sh, qk, ku, kind, sm);
         __syncthreads();
     }
     ns_rhs_to_fp64<NT>(s, c0, qk, sm);
@@ -1795,12 +1876,12 @@ template <int D, int NT, bool ALL_TEAMS = false>
 __device__ bool ns_solve(const SolveArgs& a, const Shape& sh, int j, int q, int q1,
                          const NullSmem& sm, int kind) {
     const int tid = threadIdx.x, n = sh.n, M = sh.M;
-    const int icoef = ns_coef<D>(sh), fs = ns_bits(icoef);
+    const KernelUnits ku = ns_units<D>(sh.m, kind);
     const int gs = ns_g_shift(sh.ell, kind);
-    const int eg_min = fs - 3;  // f1 fits the unit of its products (ns_product_c)
+    const int eg_min = ku.eF - ku.eA - 1;  // f1 fits the unit of its products (ns_product_c)
     if (tid == 0) {
         s_ns_eb = 0;
-        s_ns_ec = sh.m - 2;  // A22 (scale 2^m) fits the unit of the sums
+        s_ns_ec = ku.eA - 2;  // A22 (scale 2^eA) fits the unit of the sums
         s_ns_saddle = 0;
     }
     ns_coordinates<D, NT>(a, sh, j, sm);
@@ -1812,20 +1893,25 @@ __device__ bool ns_solve(const SolveArgs& a, const Shape& sh, int j, int q, int 
 #pragma unroll 1
     for (int t = tid; t < n; t += NT) sm.pos[sm.order[t]] = t;
     __syncthreads();
-    ns_pairs<D, NT>(sh, q1, icoef, fs, sm);
+    ns_pairs<D, NT>(sh, q1, ku, sm);
     __syncthreads();
     if (kind == 2) {
         double nv[D];
         scaled_normal<D>(a, j, nv);
 #pragma unroll 1
-        for (int u = tid; u < n; u += NT) {
+        for (int u = tid; u < n; u += NT) {  // (the center is the origin: node 0)
             const int p = sm.pos[u];
+            double dot = 0.0;
+            for (int c = 0; c < D; ++c)
+                dot = fma(__ll2double_rn(sm.xi[u * D + c]) * (1.0 / (1ll << kCoordBits)), nv[c], dot);
+            const long long f = ns_rhs_fixed(ns_powers<D>(sm.xi + u * D, sm.xi, sh.m, ku.beta), sh.m, ku);
             fixed(sm.X)[p < M ? p : sm.x2 + p - M] =
-                to_fixed(neumann_at<D>(sh, nv, u, sm.xi + u * D), p < M ? sh.m + sm.eg[0] + kSumUnit - 1 : sh.m - 2 + fs - kPowerBits);
+                to_fixed(-dot * from_fixed(f, ku.eF - kPowerBits),
+                         p < M ? ku.eA + sm.eg[0] + kSumUnit - 1 : ku.eF - kPowerBits);
         }
         __syncthreads();
     }
-    return ns_columns<D, NT, ALL_TEAMS>(a, sh, j, 0, q1, sh.m - 2 + fs, sm, kind) ||
+    return ns_columns<D, NT, ALL_TEAMS>(a, sh, j, 0, q1, ku, sm, kind) ||
            saddle_columns<D, NT>(a, sh, j, 0, q1, sm, kind);
 }
 
@@ -1855,17 +1941,16 @@ __device__ __forceinline__ bool ns_solve_chunk(const SolveArgs& a, const Shape& 
         return ok;
     }
     const int n = sh.n, M = sh.M;
-    const int icoef = ns_coef<D>(sh), fs = ns_bits(icoef);
+    const KernelUnits ku = ns_units<D>(sh.m, 0);
 #pragma unroll 1
     for (int e = threadIdx.x; e < n * qk; e += NT) {
         const int c = small_div(e, n), u = e - c * n, p = sm.pos[u], t = sm.cols[c0 + c];
-        long long pm2 = 0, pm;
-        if (u != t) ns_powers<D>(sm.xi + u * D, sm.xi + t * D, sh.m, &pm2, &pm);
-        const long long f = ns_rhs_fixed(pm2, icoef, fs);
-        fixed(sm.X)[c * sm.ldx + (p < M ? p : sm.x2 + p - M)] = p < M ? shift_fixed(f, fs - 3 - sm.eg[c0 + c]) : f;
+        const long long f = ns_rhs_fixed(ns_powers<D>(sm.xi + u * D, sm.xi + t * D, sh.m, ku.beta), sh.m, ku);
+        fixed(sm.X)[c * sm.ldx + (p < M ? p : sm.x2 + p - M)] =
+            p < M ? shift_fixed(f, ns_f1_shift(ku, sm.eg[c0 + c])) : f;
     }
     __syncthreads();
-    ns_columns<D, NT, false>(a, sh, j, c0, qk, sh.m - 2 + fs, sm, 0);
+    ns_columns<D, NT, false>(a, sh, j, c0, qk, ku, sm, 0);
     ns_lebesgue<NT>(sh, c0, qk, sm);
     return true;
 }

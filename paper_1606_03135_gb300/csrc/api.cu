@@ -527,21 +527,25 @@ int plan_impl(const double* nodes, int64_t N, int d, int n, int ell, int m,
                           : o.refine == RBFFD_REFINE_ALL           ? 0
                                                                    : RBFFD_REFINE_MIN_K;
         // Layouts to try.  LDL^T solves systems of one shape in the null space of the constraints
-        // when r^m is conditionally definite there (ell >= (m - 1) / 2) and the fixed-point forms
-        // are as accurate as the saddle-point factorization against a double-double solve: up to
-        // r^7 and degree 5 the norms of their errors over a set's rows are 0.5 to 1.0 times its
-        // (1.3 on a set whose largest error is one row's).  At degree 6 and above (the constraints'
-        // pivots get small) and at r^9 and above (r^m spans more of the 58 bits) they are larger.
-        // Degree 5 with K < 100 (2D; not refined) keeps the saddle-point path although the null
-        // space is faster there (n = 43, N = 30k, delta 0.6: 1.6 against 2.55 ms): on sets with
-        // nearly coincident nodes that path's own error passes 1e-9 of the matrix's norm, so no
-        // other solver reproduces its matrix to that.  Large systems (K >= 100, which refine) with
-        // n > 3 M are left out as well: S is nearly the whole matrix there (n = 128, M = 21: 5.0 ms
-        // against 5.35).  Those, plans of several shapes and systems too large for this layout
+        // when r^m is conditionally definite there (ell >= (m - 1) / 2), where this is as accurate
+        // as the saddle-point factorization against an 80-bit solve (up to r^7 and degree 5: the
+        // errors' medians and means over a set's rows are 0.8 to 1.1 times its; not examined above)
+        // and where it is faster (traversal and own-stencil kernels, saddle point / null space):
+        // - degree 1 up to n = 5 M (2D n = 15, 3D n = 20: 0.97 to 1.2; n = 25: 0.89 to 1.15; above,
+        //   S is nearly the whole system);
+        // - K >= 100 (plans that refine) up to n = 3 M (n = 128, M = 21: 5.0 ms against 5.35) and
+        //   n + q = 5.5 M with q columns, which make the tableau (M = 35: n = 96, q = 95 1.02 to
+        //   1.14; n = 100, q = 99 0.93 to 1.04; n = 105, q = 103 0.90).
+        // Degree 5 with K < 100 (2D) keeps the saddle-point path although the null space was faster
+        // there (n = 43, N = 30k, delta 0.6: 1.6 against 2.55 ms): on sets with nearly coincident
+        // nodes both are 1e-9 of the matrix's norm off, each its own way, and such plans keep the
+        // matrix they had.  Those, plans of several shapes and systems too large for this layout
         // factor the saddle-point matrix.
         const bool large = p->K >= RBFFD_REFINE_MIN_K;
+        const int M = p->K - n;
         const bool null_space = ldlt && one_shape && 2 * ell + 1 >= m && m <= 7 &&
-                                (large ? ell <= 5 && n <= 3 * (p->K - n) : ell <= 4);
+                                (large ? ell <= 5 && n <= 3 * M && 2 * (n + qmax) <= 11 * M
+                                       : ell <= 4 && (ell > 1 || n <= 5 * M));
         const int qcap0 = p->qcap;
         for (p->lay = null_space ? kLayNull : (ldlt ? kLayPacked : kLayFull);; p->lay = kLayPacked) {
             for (p->qcap = qcap0;; --p->qcap) {

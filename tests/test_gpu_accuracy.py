@@ -11,6 +11,7 @@ from paper_1606_03135_gb300 import nodesets as NS
 from paper_1606_03135_gb300 import rbffd as R
 from tests.test_gpu_degenerate import lattice
 from tests.test_gpu_flat import errors
+from tests.test_gpu_nullspace import check
 from tests.test_gpu_parity import gpu_run
 
 torch = pytest.importorskip("torch")
@@ -28,3 +29,9 @@ def test_the_median_error_is_an_lu_solver_s(name, n, ell, m):
     rows = np.random.default_rng(5).choice(len(X), 120, replace=False)
     e_gpu, e_ora = errors(X, g, ref, ell, m, rows, n)
     assert np.median(e_gpu) <= 1.25 * np.median(e_ora), (np.median(e_gpu), np.median(e_ora))
+
+
+@pytest.mark.parametrize("d,n,ell,m,delta", [(2, 15, 1, 3, 0.3), (2, 16, 1, 3, 0.3), (3, 20, 1, 3, 0.3),
+                                             (3, 21, 1, 3, 0.3), (3, 105, 4, 7, 0.03), (3, 105, 4, 7, 0.4)])
+def test_shapes_on_both_sides_of_the_layout_rule(d, n, ell, m, delta):
+    check(NS.jittered_grid(14 if d == 2 else 7, d, amp=0.3, seed=n), n, ell, m, delta)

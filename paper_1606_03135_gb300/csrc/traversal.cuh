@@ -1433,8 +1433,8 @@ __device__ __noinline__ bool ns_eliminate_fp64(const SolveArgs& a, const Shape& 
 // 80-bit solve (r^7, this / r^m itself / the saddle-point layout): disk, degree 3, n = 21, 2.3e-13 /
 // 3.1e-13 / 2.3e-13; degree 4, n = 31, 1.6e-12 / 2.4e-12 / 1.8e-12; lattice, degree 4, 3.9e-13 /
 // 1.5e-12 / 4.0e-13; ball, degree 4, n = 71, 2.2e-12 / 2.4e-12 / 2.5e-12; degree 5, n = 113, 1.2e-11 /
-// 1.5e-11 / 1.3e-11.  It costs 30 instructions a pair and saves the products of lower limbs that the
-// sums needed before (552 plans: the same time, geometric mean of the ratios 1.00).
+// 1.5e-11 / 1.3e-11.  It costs about 30 instructions a pair and saves the products of lower limbs that
+// the sums needed before (552 plans: the same time, geometric mean of the ratios 1.00).
 struct KernelUnits {
     int beta;    // of 256
     int eA, eF;  // |phi| < 2^eA, |f| < 2^eF
@@ -1462,6 +1462,11 @@ struct PairPowers {
     int delta;
 };
 
+// a z 2^-64 for z >= 0 (__mul64hi would look at the sign of z too).
+__device__ __forceinline__ long long mul_by(long long a, long long z) {
+    return (long long)__umul64hi((unsigned long long)a, (unsigned long long)z) - ((a >> 63) & z);
+}
+
 // The squared distance in u is formed in FP64 without FMA, rounded as the oracle's: the weights are as
 // far from an exact solve as that rounding puts every FP64 solver's, and so near to theirs.  In p it
 // has to be exact, or p would be no polynomial: z and the exact square differ by delta in 2^-63, a
@@ -1487,20 +1492,20 @@ __device__ __noinline__ PairPowers ns_powers(const long long* xa, const long lon
     const unsigned long long b = (unsigned long long)__double_as_longlong(r2);
     const int e = (int)(b >> 52) - 1023 - 2 * kCoordBits, odd = e & 1;  // r^2 = w 4^h, w in [1, 4)
     const unsigned long long N = ((b & 0xFFFFFFFFFFFFFull) | (1ull << 52)) << (10 + odd);  // w 2^62
-    const unsigned long long zr = b == 0ull ? 0ull : N >> min(2 + odd - e, 63) << 1;
+    const unsigned long long zr = N >> min(2 + odd - e, 63) << 1;
     PairPowers o;
     o.delta = (int)((unsigned)zr - exact);
     o.z = (long long)min(zr, 0x7fffffffffffffffull);
     const unsigned long long u =
-        b == 0ull ? 0ull : ((unsigned long long)sqrt_core(N) << 2) >> min(1 - ((e - odd) >> 1), 63);
+        ((unsigned long long)sqrt_core(N) << 2) >> min(1 - ((e - odd) >> 1), 63);
     long long p = (long long)u - ((long long)beta << (kPowerBits - 8));
     const int k = (m - 3) / 2;
-#pragma unroll 1
-    for (int s = 0; s < k; ++s) p = __mul64hi(p << 1, o.z);
+    if (k > 0) p = mul_by(p << 1, o.z);
+    if (k > 1) p = mul_by(p << 1, o.z);
     o.pk = p;
     // beta (z^(k+1) - its exact value) = beta (k + 1) z^k delta, z^k with 12 bits
     const int zt = (int)(o.z >> 51), zk = k == 0 ? 4096 : (k == 1 ? zt : zt * zt >> 12);
-    o.phi = __mul64hi(p << 1, o.z) + ((long long)o.delta * (beta * (k + 1) * zk) >> 21);
+    o.phi = mul_by(p << 1, o.z) + ((long long)o.delta * (beta * (k + 1) * zk) >> 21);
     return o;
 }
 
@@ -1512,7 +1517,7 @@ __device__ __forceinline__ long long scale_by(long long v, int c, int s) {
 // f of a pair, in 2^(eF - kPowerBits): c1 u z^k - beta c3 z^k = c1 pk + beta (c1 - c3) z^k, and as above
 // for the exact z^k of p.
 __device__ __forceinline__ long long ns_rhs_fixed(const PairPowers& o, int m, const KernelUnits& ku) {
-    const long long zk = m == 3 ? 1ll << kPowerBits : (m == 5 ? o.z >> 1 : __mul64hi(o.z, o.z));
+    const long long zk = m == 3 ? 1ll << kPowerBits : (m == 5 ? o.z >> 1 : (long long)__umul64hi(o.z, o.z));
     const int zt = (int)(o.z >> 51), dz = m == 3 ? 0 : (m == 5 ? 4096 : 2 * zt);  // k z^(k-1)
     const long long fix = (long long)o.delta * (ku.beta * ku.c3) * dz >> 21;
     return scale_by(o.pk, ku.c1, ku.fs) + scale_by(zk, (ku.c1 - ku.c3) * ku.beta, ku.fs + 8) + (fix >> ku.fs);

@@ -56,6 +56,7 @@ struct rbffd_plan_s {
     int qcap = 0, stride = 0;
     LaunchPlan lp;
     int lay = kLayPacked;           // layout of the local systems
+    bool lattice = false;           // a good part of the nodes lies inside lattices
     int refine_min_K = 0x7fffffff;  // systems with K >= this are refined
     long long rs_doubles = 0, rs_stride = 0;  // refinement scratch: size, per traversal CTA
     int rs_x0 = 0;                  // offset of the first solution within a slot
@@ -501,6 +502,7 @@ int plan_impl(const double* nodes, int64_t N, int d, int n, int ell, int m,
     }
     if (p->h_ctr.status) { rc = p->h_ctr.status; goto fail; }
     p->max_ball = p->h_ctr.max_ball;
+    p->lattice = like ? like->lattice : 16ll * p->h_ctr.n_lattice > N;
     {
         // device bytes the traversal and CSR arrays will take (same layout as rbffd_assemble)
         const size_t S = (size_t)p->total_slots, Nz = (size_t)N, nz = (size_t)n;
@@ -536,6 +538,10 @@ int plan_impl(const double* nodes, int64_t N, int d, int n, int ell, int m,
         // - K >= 100 (plans that refine) up to n = 3 M (n = 128, M = 21: 5.0 ms against 5.35) and
         //   n + q = 5.5 M with q columns, which make the tableau (M = 35: n = 96, q = 95 1.02 to
         //   1.14; n = 100, q = 99 0.93 to 1.04; n = 105, q = 103 0.90).
+        // At the edges of lattices the constraints depend on each other, and such stencils are solved
+        // as saddle-point systems in global memory.  Plans of lattices (the inside of a 3D one of
+        // 30^3 nodes is two thirds of it at n = 45, where it took three times as long) keep the
+        // saddle-point layout but for 2D ones with n >= 2 M, whose edges are few.
         // Degree 5 with K < 100 (2D) keeps the saddle-point path although the null space was faster
         // there (n = 43, N = 30k, delta 0.6: 1.6 against 2.55 ms): on sets with nearly coincident
         // nodes both are 1e-9 of the matrix's norm off, each its own way, and such plans keep the
@@ -545,7 +551,8 @@ int plan_impl(const double* nodes, int64_t N, int d, int n, int ell, int m,
         const int M = p->K - n;
         const bool null_space = ldlt && one_shape && 2 * ell + 1 >= m && m <= 7 &&
                                 (large ? ell <= 5 && n <= 3 * M && 2 * (n + qmax) <= 11 * M
-                                       : ell <= 4 && (ell > 1 || n <= 5 * M));
+                                       : ell <= 4 && (ell > 1 || n <= 5 * M)) &&
+                                (!p->lattice || (d == 2 && n >= 2 * M));
         const int qcap0 = p->qcap;
         for (p->lay = null_space ? kLayNull : (ldlt ? kLayPacked : kLayFull);; p->lay = kLayPacked) {
             for (p->qcap = qcap0;; --p->qcap) {

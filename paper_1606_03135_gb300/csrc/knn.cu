@@ -728,6 +728,13 @@ __global__ void __launch_bounds__(256) k_knn(const double* __restrict__ X, int N
             ball_len[q] = blen;
             atomicMax(&ctr->max_ball, blen);
         }
+        // Inside a lattice the neighbours come in pairs of equal distance (a lattice is symmetric about
+        // its nodes): the D nearest pairs, to 2^-30, one per lane.
+        if (nq > 2 * D) {
+            const int t = 2 * min(lane, D - 1) + 1;
+            const bool pair = rk[ord ? ord[t + 1] : t + 1] - rk[ord ? ord[t] : t] < 1ull << 22;
+            if (__all_sync(0xffffffffu, pair) && lane == 0) atomicAdd(&ctr->n_lattice, 1);
+        }
         for (int t = 1 + lane; t < blen; t += 32) {
             const int i = ri[ord ? ord[t] : t];
             if (i > q) atomicAdd(&indeg[i], 1);

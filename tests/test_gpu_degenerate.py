@@ -72,7 +72,7 @@ def test_lattices_are_solved_like_saddle_point_systems(d, side, n, ell, m):
     assert np.abs(a).max() <= 100.0 * np.abs(b).max()
 
 
-@pytest.mark.parametrize("d,side,n,ell,delta", [(2, 30, 25, 4, 0.4), (3, 9, 45, 3, 0.3), (3, 8, 113, 5, 0.5)])
+@pytest.mark.parametrize("d,side,n,ell,delta", [(2, 30, 25, 4, 0.4), (3, 9, 45, 3, 0.3), (3, 8, 64, 4, 0.5)])
 def test_lattices_in_teams_and_chunks_are_bitwise_equal(d, side, n, ell, delta):
     X = lattice(side, d)
     for mode in (R.STAB_OFF, R.STAB_FALLBACK):
@@ -114,3 +114,45 @@ def test_nodes_on_a_line_stay_singular():
         with pytest.raises(R.RbffdError) as e:
             p.assemble()
         assert e.value.code == R.ESINGULAR
+
+
+@pytest.mark.parametrize("n,ell,m", [(27, 3, 7), (45, 3, 7), (30, 3, 7), (71, 4, 7), (113, 5, 7)])
+def test_lattice_patches_in_other_node_sets(n, ell, m):
+    """Too few lattice nodes for the plan to leave the null-space layout: their stencils alone are
+    solved as saddle-point systems, at delta = 1 and with several columns."""
+    side = 7
+    X = np.concatenate([lattice(side, 3) + 10.0, NS.ball3d(6000, seed=6)])
+    N, K = len(X), side ** 3
+    g = gpu_run(X, n, ell, m, 1.0)
+    assert g["stats"]["n_singular"] == 0
+    ref = saddle(X, n, ell, m, 1.0)
+    kind = np.array([constraints(X, g["nbr"][i], ell) for i in range(K)])
+    assert (kind[:, 0] > 0).sum() > 0
+    a = g["val"].reshape(N, n)[:-1]
+    b = np.array([ref["val"][ref["row_ptr"][i]:ref["row_ptr"][i + 1]] for i in range(N - 1)])
+    assert np.isfinite(a).all() and not np.array_equal(a, b)
+    err = np.linalg.norm(a - b, axis=1) / np.linalg.norm(b, axis=1)
+    assert err[:K][kind[:, 0] == 0].max(initial=0.0) < 1e-9 and err[K:].max() < 1e-9
+    assert err[:K][(kind[:, 0] > 0) & (kind[:, 1] == 1)].max(initial=0.0) < 2e-8
+    assert np.abs(a).max() <= 100.0 * np.abs(b).max()
+    for mode in (R.STAB_OFF, R.STAB_FALLBACK):
+        p = gpu_run(X, n, ell, m, 0.4, mode)
+        assert p["stats"]["n_singular"] == 0 and np.isfinite(p["val"]).all()
+        for kw in (dict(team=32, rhs_chunk=3), dict(team=256), dict(team=512, rhs_chunk=5)):
+            q = gpu_run(X, n, ell, m, 0.4, mode, **kw)
+            for key in ("val", "owner", "lam_row"):
+                assert np.array_equal(p[key], q[key]), (key, kw)
+
+
+def test_plans_of_lattices_have_the_saddle_point_layout():
+    """The same bits as a plan of two shapes has, from a new plan and from one of another delta; turned
+    and far from the origin too."""
+    rot = np.linalg.qr(np.random.default_rng(1).normal(size=(3, 3)))[0]
+    for X in (lattice(12, 3), lattice(12, 3) * np.array([1.0, 1.7, 2.3]) + 1000.0, lattice(12, 3) @ rot):
+        t = torch.from_numpy(X).cuda()
+        b = saddle(X, 45, 3, 7, 1.0)
+        with R.Plan(t, 45, 3, 7, 0.5) as base, base.with_delta(1.0) as p:
+            p.assemble()
+            val = p.export()[2]
+        assert np.array_equal(val[:45 * (len(X) - 1)], b["val"][:45 * (len(X) - 1)])
+        assert np.array_equal(val, gpu_run(X, 45, 3, 7, 1.0)["val"])

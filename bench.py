@@ -121,26 +121,30 @@ class ClockSampler:
                 "reasons": sorted(reasons), "samples": len(sm)}
 
 
-def kernel_source_hash(path):
-    """sha256 (16 hex digits) of a CUDA source with its comments and blank space removed, so
+def kernel_source_hash(*paths):
+    """sha256 (16 hex digits) of CUDA sources with their comments and blank space removed, so
     that a comment edit does not invalidate counters taken from the same kernel code."""
     import re
-    src = open(path).read()
+    src = "\n".join(open(p).read() for p in paths)
     src = re.sub(r"/\*.*?\*/", "", src, flags=re.S)
     src = re.sub(r"//[^\n]*", "", src)
     src = "\n".join(line.strip() for line in src.splitlines() if line.strip())
     return hashlib.sha256(src.encode()).hexdigest()[:16]
 
 
+# the sources that the traversal kernels are made of
+TRAVERSAL_SOURCES = ("traversal.cuh", "nullspace.cuh", "fp64_int.cuh", "rbffd_internal.cuh")
+
+
 def _traffic_entry(workload):
     """DRAM traffic of the traversal kernel on `workload` from the committed ncu summary, if
     the kernel source is unchanged since it was captured."""
     path = os.path.join(ROOT, "profiles", "traversal_traffic.json")
-    src = os.path.join(ROOT, "paper_1606_03135_gb300", "csrc", "assemble.cu")
+    csrc = os.path.join(ROOT, "paper_1606_03135_gb300", "csrc")
     try:
         rec = json.load(open(path))
-        h = kernel_source_hash(src)
-        if rec.get("assemble_cu_code_sha256_16") == h and rec.get("workload") == workload:
+        h = kernel_source_hash(*(os.path.join(csrc, f) for f in TRAVERSAL_SOURCES))
+        if rec.get("traversal_code_sha256_16") == h and rec.get("workload") == workload:
             return rec
     except (OSError, ValueError):
         pass

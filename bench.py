@@ -138,7 +138,7 @@ TRAVERSAL_SOURCES = ("traversal.cuh", "nullspace.cuh", "fp64_int.cuh", "rbffd_in
 
 def _traffic_entry(workload):
     """DRAM traffic of the traversal kernel on `workload` from the committed ncu summary, if
-    the kernel source is unchanged since it was captured."""
+    the kernel's sources are unchanged since it was captured."""
     path = os.path.join(ROOT, "profiles", "traversal_traffic.json")
     csrc = os.path.join(ROOT, "paper_1606_03135_gb300", "csrc")
     try:
@@ -149,6 +149,33 @@ def _traffic_entry(workload):
     except (OSError, ValueError):
         pass
     return None
+
+
+# What a roofline entry keeps inside `configs` (the headline's is whole, and a run of one --workload
+# prints its own whole), so that the line stays below the 8 KB or so that readers of a run's output keep.
+ROOFLINE_SHORT = ("bound", "achieved", "frac", "frac_of_measured_dfma", "kernel_ms")
+
+
+def compact(line):
+    """The line as printed: floats to 6 significant digits (5 in the further configs); in those,
+    roofline entries down to ROOFLINE_SHORT (peak and unit are the headline's), and left out beside an
+    `fp64_frac`, which says the same."""
+    def walk(v, inside):
+        if isinstance(v, dict):
+            out = {}
+            for k, x in v.items():
+                if inside and k == "roofline" and isinstance(x, dict):
+                    if "fp64_frac" in v:
+                        continue
+                    x = {r: x[r] for r in ROOFLINE_SHORT if r in x}
+                out[k] = walk(x, inside or k == "configs")
+            return out
+        if isinstance(v, (list, tuple)):
+            return [walk(x, inside) for x in v]
+        if isinstance(v, float) and math.isfinite(v):
+            return float(f"{v:.5g}" if inside else f"{v:.6g}")
+        return v
+    return walk(line, False)
 
 
 def max_over_ranks(x: float, device="cpu") -> float:
@@ -436,11 +463,9 @@ def run_sweep(args, name, dev, world=1, e2e=True, steps=None, warmup=None):
                                       f"{w['timestep_c']:.3g}"} if bcw is not None else {}),
                       "l2": "flushed between timed steps (256 MB write)",
                       "plans": ("each delta's own kNN" if fresh else
-                                "one kNN per step: the first delta's plan searches the stencils, "
-                                "the others copy them and recompute their balls "
+                                "one kNN per step, the later deltas' stencils are copies "
                                 "(rbffd_plan_delta)") +
-                               "; built on a side stream beside the previous delta's assembly "
-                               "(per_delta ms_stencils of later deltas include that overlap)",
+                               "; on a side stream beside the previous assembly",
                       "schedule": ({str(k): v for k, v in sched.items()}
                                    if not args.no_autotune else "library default"),
                       "deltas_concurrent": bool(conc), "elastic": elastic},
@@ -741,7 +766,7 @@ def run_gpu(args):
         line["cpu_baseline"] = cpu_baseline_entry()
     line["bench_wall_s"] = time.perf_counter() - t_start
     if rank == 0:
-        print(json.dumps(line), flush=True)
+        print(json.dumps(compact(line), separators=(",", ":")), flush=True)
     if world > 1:
         import torch.distributed as dist
         dist.destroy_process_group()

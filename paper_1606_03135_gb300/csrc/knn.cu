@@ -796,7 +796,7 @@ static size_t round256(size_t b) { return (b + 255) & ~size_t(255); }
 
 size_t grid_scratch_bytes(int N, int D, int ncell_max) {
     size_t b = round256(sizeof(GridParams)) + round256(sizeof(BBoxAcc));
-    b += 3 * round256((size_t)(ncell_max + 1) * sizeof(int));  // count, start, one to spare
+    b += 2 * round256((size_t)(ncell_max + 1) * sizeof(int));  // count, start
     b += 2 * round256((size_t)N * sizeof(int));                // cell_of, sorted_idx
     b += round256((size_t)N * D * sizeof(double));             // sorted_X
     b += round256((size_t)N * D * sizeof(float));              // sorted_Xf (FP32 screen)

@@ -67,7 +67,7 @@ def estimate_bytes(N: int, d: int, n: int, delta: float, ell: int = None) -> int
     per SM); without `ell` that is assumed.  The exact figure is known after the plan (rbffd_stats: plan_bytes
     + assemble_bytes) and never exceeds this."""
     ball = 1 if delta >= 1.0 else n
-    plan = N * (d * 8 + n * 4 + 8 + 4 + 4 + 8) + (2 * N + 64) * 12 + N * (8 + 8 * d)
+    plan = N * (d * 8 + n * 4 + 8 + 4 + 4 + 8) + (2 * N + 64) * 8 + N * (8 + 8 * d)
     asm = N * (4 * 6 + 2 + n * 12 + 16) + N * ball * (n * 8 + 9)
     refined = ell is None or n + math.comb(ell + d, d) >= 100
     return int(plan + asm + (9 << 20) + ((200 << 20) if refined else 0))

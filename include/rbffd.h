@@ -47,9 +47,12 @@ extern "C" {
 
 /* Factorization of the local symmetric saddle-point system (§4.1, §4.3 "one matrix
  * decomposition").  LDLT: symmetric indefinite LDL^T with Bunch-Kaufman pivoting,
- * (1/3) K^3 flops, or, for plans of one stencil shape with r^7 or below, 2 degree + 1 >= the
- * exponent, and degree up to 4, or K >= 100, n <= 3 M and degree up to 5, an LDL^T of the system
- * reduced to the null space of the polynomial constraints (as accurate, most of it in fixed point);
+ * (1/3) K^3 flops, or, for plans of one stencil shape with r^7 or below and 2 degree + 1 >= the
+ * exponent, an LDL^T of the system reduced to the null space of the polynomial constraints (as
+ * accurate, most of it in fixed point).  That is taken for degree 1 up to n = 5 M, degrees 2 to 4
+ * and, where K >= 100, degrees up to 5 with n <= 3 M and n + q <= 5.5 M for balls of up to q nodes;
+ * not on lattices in 3D, nor in 2D with n < 2 M.  Stencils that the null space cannot solve
+ * (dependent constraints, nodes nearer than rounding) take the saddle-point factorization one by one.
  * LU: partial-pivot LU, (2/3) K^3 flops.  Same weights up to rounding. */
 #define RBFFD_FACTOR_LDLT 0
 #define RBFFD_FACTOR_LU 1
@@ -104,11 +107,14 @@ typedef struct {
                            memory before the factorization: one full K x K copy per resident
                            CTA; in the null space its entries are formed again) and the
                            correction is solved with
-                           the stored factors (about 4 K^2 flops per refined column).  With a
-                           Lebesgue test (SEQ, FALLBACK) a column whose first Lebesgue value
+                           the stored factors (about 4 K^2 flops per refined column).  Null-space
+                           systems refine every column.  In the others, with a
+                           Lebesgue test (SEQ, FALLBACK), a column whose first Lebesgue value
                            exceeds the test's reference by more than 2^-10 of it is not
                            refined: it fails the test either way and its weights are
                            discarded; the matrix is the same as with every column refined.  The
+                           few systems that a null-space plan solves as saddle-point systems
+                           (see factor) are not refined.  The
                            traversal's 96- and 128-thread teams have no refinement step, so
                            forcing them (opts.team) on a plan that refines is RBFFD_EINVAL.
                            RBFFD_FACTOR_LU is never refined.  Other values: RBFFD_EINVAL */
@@ -302,7 +308,8 @@ int rbffd_stencils_noalloc(const double* nodes, int64_t N, int d, int n, double 
  *   bc       host array [N]: 0 interior, 1 Dirichlet, 2 Neumann (other values: RBFFD_EINVAL);
  *            NULL removes the boundary
  *   normals  host array [N][d] row-major: the unit outward normal of each Neumann node (other
- *            rows are ignored); may be NULL when no node is Neumann (else RBFFD_EINVAL);
+ *            rows are ignored; one of another length scales its row); may be NULL when no node is
+ *            Neumann (else RBFFD_EINVAL);
  *            non-finite entries of Neumann rows: RBFFD_EINVAL
  * Takes effect at the next rbffd_assemble: the overlapped traversal then runs over the
  * interior only (a boundary node is never a center and never in a retention set, so

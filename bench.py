@@ -296,9 +296,8 @@ def roofline_entry(stats, kernel_ms, kernel, share=None, traffic=None, factor_lu
     flops_executed: (1/3) K^3 per LDL^T factorization ((2/3) K^3 for LU) + 2 K^2 per solved
     column (every retained node, kept or rejected); flops_survey: the cost model's
     (2/3) K^3 + 2 K^2 p.  The refinement step's work is reported beside, not counted.  Both count
-    the saddle-point factorization whatever the plan's layout: null-space plans (one stencil
-    shape, degree up to 4, or 5 from K = 100 on, r^7 or below) do most of that work in fixed point on the integer
-    pipe, so their `frac` compares with the FP64 peak but is no utilization of it."""
+    the saddle-point factorization whatever the plan's layout: null-space plans do most of that work
+    in fixed point on the integer pipe, so their `frac` compares with the FP64 peak but is no utilization of it."""
     k3 = sum(s["sum_k3"] for s in stats)
     k2c = sum(s["sum_k2_cols"] for s in stats)
     executed = (2.0 / 3.0 if factor_lu else 1.0 / 3.0) * k3 + 2.0 * k2c

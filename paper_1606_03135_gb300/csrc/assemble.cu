@@ -15,9 +15,9 @@
 //
 // Local solve (one team of 32 to 512 threads per stencil).  The (n+M) x (n+M) saddle-point
 // matrix [A P; P^T 0] of §4.1 and the q right-hand sides of the overlapped system (one per
-// solved ball member) are formed in shared memory.  Plans whose stencils have one shape with
-// degree up to 4 (5 for K >= 100) and r^7 or below solve in the null space of P^T
-// (nullspace.cuh: most of the work in fixed point on the integer pipe).  For the others the
+// solved ball member) are formed in shared memory.  Most plans of one stencil shape with r^7 or
+// below solve in the null space of P^T (nullspace.cuh: most of the work in fixed point on the
+// integer pipe; the plan's rule stands in api.cu).  For the others the
 // lower triangle is stored packed and factored as L D L^T with Bunch-Kaufman pivoting, the
 // right-hand sides carried along ((1/3) K^3 + 2 K^2 q flops); the paper's
 // partial-pivot LU of the full [A_hat | B_hat] array ((2/3) K^3 + 2 K^2 q) is the
@@ -404,10 +404,10 @@ static int pick_team(int lay, size_t smem, int force, int* nt_out, int* per_sm_o
         // Null-space solves: a warp per system while at least 12 of them share an SM (enough warps
         // to hide each other's latency, no barriers), 128 threads down to five, 256 for two to
         // four, 512 for one.  Traversal ms (32 / 128 threads): 3D ball N = 100k delta 1.0 (16 systems
-        // per SM) 8.7 / 10.9, 0.4 (9) 6.7 / 6.1, 0.2 (6) 9.0 / 6.6; 2D square N = 40k delta 1.0 (22)
-        // 1.65 / 2.50, 0.3 (12) 0.82 / 0.87.  Plans that refine (not in 128-thread teams): 64 from
-        // six systems on, else 256: 3D degree 4 N = 12k delta 1.0 (6; 64 / 256) 3.9 / 4.4, 0.4 (3)
-        // 2.6 / 1.9.
+        // per SM) 9.1 / 10.8, 0.4 (8) 7.0 / 6.1, 0.2 (6) 9.0 / 6.5; 2D square N = 40k delta 1.0 (16)
+        // 1.68 / 2.40, 0.3 (12) 0.86 / 0.85.  Plans that refine (not in 128-thread teams): 64 from
+        // six systems on, else 256: 3D degree 4 N = 12k delta 1.0 (6; 64 / 256) 3.8 / 4.1, 0.4 (3)
+        // 2.5 / 1.8.
         int per_sm = 0;
         if ((rc = occ(32, &per_sm))) return rc;
         const bool many = refined ? per_sm >= 6 : per_sm >= 5;

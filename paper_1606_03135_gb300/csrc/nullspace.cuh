@@ -149,9 +149,9 @@ constexpr int kSumUnit = 2 * kLimbBits - 2 * kFixBits;  // -60
 // Row stride of the tableau and of C in 8-byte words: an odd multiple of 16 bytes, so 16-byte
 // loads of consecutive rows hit distinct banks.  Systems of one column run in teams of one warp,
 // for which more of them per SM count for more than a two-way conflict, so there the pad is left
-// out (3D, M = 20, n = 45, N = 100k, delta = 1: 16 systems per SM instead of 14, 9.2 -> 8.7 ms;
-// with it left out at delta 0.4 and 0.2 too, 128-thread teams took 2% longer) unless rows would
-// then share a quarter of the banks (2D, M = 15: 1.60 -> 1.90 ms).
+// out (3D, M = 20, n = 45, N = 100k, delta = 1: 16 systems per SM instead of 14, 9.1 ms instead of
+// 10.0; with it left out at delta 0.4 and 0.2 too, 128-thread teams took 1% longer) unless rows would
+// then share a quarter of the banks (2D, M = 15: 1.95 ms instead of 1.68).
 __host__ __device__ __forceinline__ int ns_ldm(int M, int qmax) {
     const int e = (M + 1) / 2;
     return 2 * (qmax > 1 || (e & 3) == 0 ? e | 1 : e);

@@ -1636,13 +1636,12 @@ __device__ __forceinline__ void ns_rhs_to_fp64(int s, int c0, int qk, const Null
 // rho = f - A w in FP64 with the entries of A and f formed as the saddle-point systems form them
 // (correctly rounded coordinates, no FMA in the squared distances), then S dv = rho_other -
 // B rho_basic with the stored factors and w_basic -= B^T dv.  (The constraints hold by construction
-// and are left alone.)  Below a pivot span of 2^10 the unrefined weights are as close to a
-// double-double solve as refined ones (means over 60 stencils, unrefined / refined / refined
-// saddle-point solve: 3D ball, degree 5, 4.1e-12 / 3.9e-12 / 4.0e-12), from there on refinement
-// halves their error (clustered cube, degree 5, spans of 2^10 to 2^12: 9.5e-11 / 4.1e-11 /
-// 4.2e-11).  So in plans that refine (K >= 100) systems whose pivots span at least 2^10 are refined
-// (7% of the ball's, three quarters of the cube's), or every system with a.refine_all.  gw: scratch
-// of 2 n words per column and n D words.
+// and are left alone.)  In plans that refine (K >= 100) systems whose pivots span at least 2^10 are
+// refined (7% of the ball's, three quarters of the clustered cube's), or every system with
+// a.refine_all.  Below that the unrefined weights are as good (ball, degree 5, n = 113, means over 190
+// rows against an 80-bit solve, all refined from 2^10 on / none / the saddle-point layout: 1.84e-11 /
+// 1.82e-11 / 1.97e-11); clustered sets need it (cube, degree 5, n = 90: 2.1e-10 / 8.7e-10 / 1.8e-10).
+// gw: scratch of 2 n words per column and n D words.
 constexpr int kNullRefineLog2 = 10;
 
 template <int D, int NT>

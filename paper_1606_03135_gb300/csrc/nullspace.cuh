@@ -34,7 +34,7 @@ constexpr int kPowerBits = 62;  // of phi and of f, which are not operands of pr
 
 // The conversions and dot products below that are used in several places are functions of their
 // own, loops are not unrolled beyond what hides their latency, and quotients of small integers take
-// an FP32 reciprocal: the kernels run the phases of up to 22 systems side by side on an SM, and with
+// an FP32 reciprocal: the kernels run the phases of up to 16 systems side by side on an SM, and with
 // everything inlined (218 KB of code) waiting for instructions took a third of the time (3D ball,
 // N = 100,000, delta = 1: 16.7 ms, against 9.9 ms at 128 KB).
 

@@ -86,7 +86,8 @@ def test_thin_stencils_in_teams_and_chunks_are_bitwise_equal(name, n, ell, delta
     X = SETS[name]()
     a = gpu_run(X, n, ell, 7, delta)
     assert a["stats"]["max_ball"] > 5 and np.isfinite(a["val"]).all()
-    for kw in (dict(team=32), dict(team=64, rhs_chunk=3), dict(team=256), dict(team=512, rhs_chunk=5)):
+    for kw in (dict(team=32), dict(team=64, rhs_chunk=3), dict(team=256), dict(team=512, rhs_chunk=5)) + \
+            ((dict(team=96), dict(team=128, rhs_chunk=2)) if n < 100 else ()):
         b = gpu_run(X, n, ell, 7, delta, **kw)
         for key in ("row_ptr", "col", "val", "owner", "is_center", "lam_row"):
             assert np.array_equal(a[key], b[key]), (key, kw)

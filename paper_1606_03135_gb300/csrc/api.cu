@@ -502,7 +502,7 @@ int plan_impl(const double* nodes, int64_t N, int d, int n, int ell, int m,
     }
     if (p->h_ctr.status) { rc = p->h_ctr.status; goto fail; }
     p->max_ball = p->h_ctr.max_ball;
-    p->lattice = like ? like->lattice : 16ll * p->h_ctr.n_lattice > N;
+    p->lattice = like ? like->lattice : 256ll * p->h_ctr.n_lattice > N;  // (1 in 16)
     {
         // device bytes the traversal and CSR arrays will take (same layout as rbffd_assemble)
         const size_t S = (size_t)p->total_slots, Nz = (size_t)N, nz = (size_t)n;

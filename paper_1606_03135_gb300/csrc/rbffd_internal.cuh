@@ -68,7 +68,7 @@ struct DevCounters {
     unsigned long long n_spec;       // speculative solves made by idle CTAs
     unsigned long long n_spec_used;  // centers that found their solve already made
     int spec_next;                   // next node an idle CTA considers for speculation
-    int n_lattice;                   // (plan) nodes whose neighbours lie in symmetric pairs
+    int n_lattice;                   // (plan) of one node in 16, those whose neighbours lie in pairs
     unsigned long long sum_k2c;      // sum over factored stencils of K^2 (columns solved)
     unsigned long long sum_k2r;      // sum over refined solves of K^2 (columns refined)
     unsigned long long pad[15];
